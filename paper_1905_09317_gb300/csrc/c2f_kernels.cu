@@ -323,33 +323,25 @@ __global__ void k_ignite(const SimJob *jobs, int32_t job) {
 }
 
 // ------------------------------------------------------------------ K3
-__device__ __forceinline__ bool plane_bit(const uint32_t *p, int32_t wpr, int32_t r, int32_t c) {
-  return (p[r * wpr + (c >> 5)] >> (c & 31)) & 1u;
-}
-
+// the least byte (16-bit minima: bytewise ones are emulated on this GPU)
 __device__ __forceinline__ uint32_t min_byte8(uint64_t v) {
-  uint32_t m = __vminu4((uint32_t)v, (uint32_t)(v >> 32));
-  m = __vminu4(m, m >> 16);
-  m = __vminu4(m, m >> 8);
-  return m & 0xFFu;
+  const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32), m8 = 0x00FF00FFu;
+  const uint32_t m = __vminu2(__vminu2(lo & m8, (lo >> 8) & m8), __vminu2(hi & m8, (hi >> 8) & m8));
+  return min(m & 0xFFFFu, m >> 16);
 }
 
-__device__ __forceinline__ int64_t axis_len(const SimJob &J, int k) {
-  return (k & 1) ? J.d_diag : J.d_orth;
-}
-
-// smallest n >= 1 with n * inc >= rem, for callers that know 64 * inc >= rem
-// (a crossing within the hour: at most 60 periods).  Six halving steps of
-// exact int64 products; a conversion of int64 operands to floating point costs
-// several times more on this GPU.
-__device__ __forceinline__ int32_t ceil_div_small(int64_t rem, int64_t inc) {
-  int32_t n = 0;   // n * inc < rem, or n = 0
-#pragma unroll
-  for (int b = 5; b >= 0; --b) {
-    const int32_t t = n + (1 << b);
-    if ((int64_t)t * inc < rem) n = t;
-  }
-  return n + 1;
+// smallest n >= 1 with n * inc >= rem, for callers that know 0 < inc, 0 < rem
+// and 64 * inc >= rem (a crossing within the hour: at most 60 periods), with
+// rem and inc both below 2^(31 + shift).  A binary32 estimate of the quotient
+// from the top bits, never more than its ceiling (inc is rounded up), then one
+// exact int64 step; the estimate falls short by two or more only when the top
+// bits of inc are few, i.e. for a last few units of a nearly finished axis.
+__device__ __forceinline__ int32_t ceil_div_small(int64_t rem, int64_t inc, int shift) {
+  const float a = (float)(uint32_t)((uint64_t)rem >> shift), b = (float)((uint32_t)((uint64_t)inc >> shift) + 1u);
+  int32_t n = (int32_t)__fdividef(a, b);
+  int64_t left = rem - (int64_t)n * inc;
+  while (left > 0) { ++n; left -= inc; }
+  return n;
 }
 
 // The frontier's two binary64 tests are kept out of line: inlined, the
@@ -388,19 +380,6 @@ __device__ __forceinline__ uint32_t warp_min(uint32_t v) {
   return __reduce_min_sync(0xffffffffu, v);   // one warp-wide reduction instruction
 }
 
-// min over the 8 lanes of this lane's group
-__device__ __forceinline__ uint32_t group_min(uint32_t v) {
-#pragma unroll
-  for (int o = 4; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-// a per-lane flag over the 8 lanes of this lane's group, as an 8-bit mask (bit k = lane k)
-__device__ __forceinline__ uint32_t group_bits(bool b) {
-  const uint32_t bal = __ballot_sync(0xffffffffu, b);
-  return (bal >> (threadIdx.x & 24)) & 0xFFu;
-}
-
 __device__ __forceinline__ uint32_t rc_pack(int32_t r, int32_t c) {
   return ((uint32_t)r << 16) | (uint32_t)c;
 }
@@ -408,13 +387,6 @@ __device__ __forceinline__ uint32_t rc_pack(int32_t r, int32_t c) {
 // a table row into L2 ahead of its use
 __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-// a 64-byte table row into this SM's L1 ahead of its use (both 32-byte
-// sectors); only for tables that no warp writes while the frontier runs
-__device__ __forceinline__ void prefetch_row_l1(const int64_t *row) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(row));
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(row + 4));
 }
 
 // chunk state, read at device scope from L2.  A relaxed load suffices: a warp
@@ -455,133 +427,68 @@ __device__ __forceinline__ void table_chunk(const SimJob &J, int32_t h, int32_t 
   __syncwarp();
 }
 
-// 32-bit atomics on words known to lie in shared memory
-__device__ __forceinline__ uint32_t atom_and_shared(uint32_t *p, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.shared.and.b32 %0, [%1], %2;"
-               : "=r"(old) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ uint32_t atom_or_shared(uint32_t *p, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.shared.or.b32 %0, [%1], %2;"
-               : "=r"(old) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ int32_t atom_exch_shared(int32_t *p, int32_t v) {
-  int32_t old;
-  asm volatile("atom.shared.exch.b32 %0, [%1], %2;"
-               : "=r"(old) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
-  return old;
-}
-
-// The replica's Available and Burned bit planes.  With WIN, a window of
-// kWinRows x (32 kWinWords) cells around the ignition cell lives in shared
+// The replica's Available bit plane, and with A5 (i) on a plane of the cells
+// that burned out by it.  With WIN, a window of kWinRows x (32 kWinWords)
+// cells of the Available plane around the ignition cell lives in shared
 // memory and the rest of the grid in global memory; without it, all in global
-// memory.  Accessors hand out a pointer to the 32-bit word holding (r, c).
+// memory.  A cell burned out by A5 (ii) needs no bit of its own: it is one
+// that ignited and has no Available neighbour.
 template <bool WIN>
 struct Planes {
-  uint32_t *sav, *sbr;   // shared-memory windows
+  uint32_t *sav;         // shared-memory window
   uint32_t *gav, *gbr;   // full planes, global memory
-  int32_t r0, w0, wpr;
+  int32_t r0, w0, rows, wpr;
   __device__ __forceinline__ bool in_win(int32_t r, int32_t w) const {
     if constexpr (WIN) return (uint32_t)(r - r0) < (uint32_t)kWinRows && (uint32_t)(w - w0) < (uint32_t)kWinWords;
     else return false;
   }
-  __device__ __forceinline__ uint32_t *avw(int32_t r, int32_t c) const {
-    const int32_t w = c >> 5;
-    if (in_win(r, w)) return sav + (r - r0) * kWinWords + (w - w0);
-    return gav + r * wpr + w;
+  // word w of row r of the Available plane (0 outside the grid)
+  __device__ __forceinline__ uint32_t word(int32_t r, int32_t w) const {
+    if ((uint32_t)r >= (uint32_t)rows || (uint32_t)w >= (uint32_t)wpr) return 0u;
+    if (in_win(r, w)) return sav[(r - r0) * kWinWords + (w - w0)];
+    return gav[r * wpr + w];
   }
-  __device__ __forceinline__ uint32_t *brw(int32_t r, int32_t c) const {
-    const int32_t w = c >> 5;
-    if (in_win(r, w)) return sbr + (r - r0) * kWinWords + (w - w0);
-    return gbr + r * wpr + w;
-  }
-  __device__ __forceinline__ bool avail(int32_t r, int32_t c) const { return (*avw(r, c) >> (c & 31)) & 1u; }
-  __device__ __forceinline__ bool burned(int32_t r, int32_t c) const { return (*brw(r, c) >> (c & 31)) & 1u; }
-  // ignition: clears the Available bit; true for the one caller that cleared it
-  // (a word of the window is changed with a shared-memory atomic, the others
-  // in global memory: an atomic on a generic address costs more than either)
-  __device__ __forceinline__ bool take(int32_t r, int32_t c) const {
+  // ignition: clears the Available bit
+  __device__ __forceinline__ void take(int32_t r, int32_t c) const {
     const uint32_t bit = 1u << (c & 31);
     const int32_t w = c >> 5;
-    if (in_win(r, w)) return (atom_and_shared(sav + (r - r0) * kWinWords + (w - w0), ~bit) & bit) != 0;
-    return (atomicAnd(gav + r * wpr + w, ~bit) & bit) != 0;
+    if (in_win(r, w)) atomicAnd(sav + (r - r0) * kWinWords + (w - w0), ~bit);
+    else atomicAnd(gav + r * wpr + w, ~bit);
   }
-  // burn-out: sets the Burned bit; true for the one caller that set it
+  // the (2 D + 1) x (2 D + 1) block of Available bits around (r, c), one row
+  // per element, bit j = column c - D + j; cells outside the grid are 0.  The
+  // common case lies in the window: a row comes out of two adjacent words by
+  // one funnel shift (bits past the last column and rows past the last one
+  // are 0 there)
+  template <int D>
+  __device__ __forceinline__ void block(int32_t r, int32_t c, uint32_t b[2 * D + 1]) const {
+    const uint32_t sh = (uint32_t)(c - D) & 31u, mask = (1u << (2 * D + 1)) - 1u;
+    const int32_t wl = (c - D) >> 5, wh = (c + D) >> 5;
+    if constexpr (WIN) {
+      if ((uint32_t)(r - D - r0) < (uint32_t)(kWinRows - 2 * D) && wl >= w0 && wh < w0 + kWinWords) {
+        const uint32_t *p = sav + (r - D - r0) * kWinWords - w0;
+#pragma unroll
+        for (int d = 0; d < 2 * D + 1; ++d)
+          b[d] = __funnelshift_r(p[d * kWinWords + wl], p[d * kWinWords + wh], sh) & mask;
+        return;
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < 2 * D + 1; ++d)
+      b[d] = __funnelshift_r(word(r - D + d, wl), word(r - D + d, wh), sh) & mask;
+  }
+  // A5 (i): has (r, c) burned out by it / the first to mark it so
+  __device__ __forceinline__ bool burned(int32_t r, int32_t c) const { return (gbr[r * wpr + (c >> 5)] >> (c & 31)) & 1u; }
   __device__ __forceinline__ bool burn(int32_t r, int32_t c) const {
     const uint32_t bit = 1u << (c & 31);
-    const int32_t w = c >> 5;
-    if (in_win(r, w)) return (atom_or_shared(sbr + (r - r0) * kWinWords + (w - w0), bit) & bit) == 0;
-    return (atomicOr(gbr + r * wpr + w, bit) & bit) == 0;
-  }
-  // the Available neighbours of (r, c) as an 8-bit mask, bit k = axis k
-  // (neighbours outside the grid are not Available)
-  __device__ __forceinline__ uint32_t avail_mask(int32_t rows, int32_t cols, int32_t r, int32_t c) const {
-    if constexpr (WIN) {
-      // the common case, as in any_avail_nbr: three window rows, funnel shifts
-      const int32_t il = ((c - 1) >> 5) - w0, ih = ((c + 1) >> 5) - w0;
-      if (c >= 1 && r >= 1 && r + 1 < rows && (uint32_t)(r - 1 - r0) < (uint32_t)(kWinRows - 2) &&
-          (uint32_t)il < (uint32_t)kWinWords && (uint32_t)ih < (uint32_t)kWinWords) {
-        const uint32_t *p = sav + (r - 1 - r0) * kWinWords;
-        const uint32_t sh = (uint32_t)(c - 1) & 31u;
-        const uint32_t up = __funnelshift_r(p[il], p[ih], sh) & 7u;                  // NW N NE
-        const uint32_t mid = __funnelshift_r(p[kWinWords + il], p[kWinWords + ih], sh) & 7u;   // W . E
-        const uint32_t dn = __funnelshift_r(p[2 * kWinWords + il], p[2 * kWinWords + ih], sh) & 7u;  // SW S SE
-        return ((mid >> 2) & 1u) | (((up >> 2) & 1u) << 1) | (((up >> 1) & 1u) << 2) | ((up & 1u) << 3) |
-               ((mid & 1u) << 4) | ((dn & 1u) << 5) | (((dn >> 1) & 1u) << 6) | (((dn >> 2) & 1u) << 7);
-      }
-    }
-    uint32_t m = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int32_t nr = r + axis_dr(q), nc = c + axis_dc(q);
-      if (nr >= 0 && nr < rows && nc >= 0 && nc < cols && avail(nr, nc)) m |= 1u << q;
-    }
-    return m;
-  }
-  // some neighbour of (r, c) is still Available
-  __device__ __forceinline__ bool any_avail_nbr(int32_t rows, int32_t cols, int32_t r, int32_t c) const {
-    if constexpr (WIN) {
-      // the common case: the 3 x 3 block lies inside the grid and the window;
-      // a row's three bits come out of two adjacent window words by one funnel
-      // shift (bits past the last column are 0 in the plane)
-      const int32_t il = ((c - 1) >> 5) - w0, ih = ((c + 1) >> 5) - w0;
-      if (c >= 1 && r >= 1 && r + 1 < rows && (uint32_t)(r - 1 - r0) < (uint32_t)(kWinRows - 2) &&
-          (uint32_t)il < (uint32_t)kWinWords && (uint32_t)ih < (uint32_t)kWinWords) {
-        const uint32_t *p = sav + (r - 1 - r0) * kWinWords;
-        const uint32_t sh = (uint32_t)(c - 1) & 31u;
-        const uint32_t up = __funnelshift_r(p[il], p[ih], sh) & 7u;
-        const uint32_t mid = __funnelshift_r(p[kWinWords + il], p[kWinWords + ih], sh) & 5u;
-        const uint32_t dn = __funnelshift_r(p[2 * kWinWords + il], p[2 * kWinWords + ih], sh) & 7u;
-        return (up | mid | dn) != 0u;
-      }
-    }
-    uint32_t words[3][2];
-    const int32_t c0 = c > 0 ? c - 1 : 0, c1 = c + 1 < cols ? c + 1 : cols - 1;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int32_t rr = r - 1 + d;
-      const bool ok = rr >= 0 && rr < rows;
-      words[d][0] = ok ? *avw(rr, c0) : 0u;
-      words[d][1] = ok ? *avw(rr, c1) : 0u;
-    }
-    bool any = false;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-#pragma unroll
-      for (int dc = -1; dc <= 1; ++dc) {
-        if (d == 1 && dc == 0) continue;
-        const int32_t cc = c + dc;
-        if (cc < 0 || cc >= cols) continue;
-        const uint32_t w = ((cc >> 5) == (c0 >> 5)) ? words[d][0] : words[d][1];
-        any |= ((w >> (cc & 31)) & 1u) != 0;
-      }
-    }
-    return any;
+    return (atomicOr(gbr + r * wpr + (c >> 5), bit) & bit) == 0;
   }
 };
+
+// three 3-bit rows around a cell (bit j = column c - 1 + j) as the 8 axes' mask, bit k = axis k
+__device__ __forceinline__ uint32_t axes_of_rows(uint32_t up, uint32_t mid, uint32_t dn) {
+  return ((mid >> 2) & 1u) | ((__brev(up) >> 28) & 0xEu) | ((mid & 1u) << 4) | ((dn & 7u) << 5);
+}
 
 // The bytes of an entry's crossing offsets: 0..sph-1 the offset in the hour
 // at which that axis reaches its neighbour's centre, kOpen an open axis with
@@ -591,40 +498,69 @@ constexpr uint32_t kOpen = 0xFEu;
 
 // the open axes of an entry (bytes that are not kNone) as an 8-bit mask
 __device__ __forceinline__ uint32_t open_axes(uint64_t c8) {
-  const uint32_t closed = byte_lsbs(__vcmpeq4((uint32_t)c8, 0xFFFFFFFFu)) |
-                          (byte_lsbs(__vcmpeq4((uint32_t)(c8 >> 32), 0xFFFFFFFFu)) << 4);
-  return ~closed & 0xFFu;
+  // a byte is below 64, 0xFE or 0xFF: closed iff bits 7 and 0 are both set
+  const uint32_t lo = (uint32_t)c8, hi = (uint32_t)(c8 >> 32);
+  return ~(byte_lsbs((lo >> 7) & lo) | (byte_lsbs((hi >> 7) & hi) << 4)) & 0xFFu;
 }
 
-// the axes of an entry crossing at offset o as an 8-bit mask (bytewise compares)
-__device__ __forceinline__ uint32_t axes_at(uint64_t c8, uint32_t o) {
-  const uint32_t oo = o * 0x01010101u;
-  return byte_lsbs(__vcmpeq4((uint32_t)c8, oo)) | (byte_lsbs(__vcmpeq4((uint32_t)(c8 >> 32), oo)) << 4);
+// the bytes of x below e (e <= 60), as the top bits of the bytes: an offset is
+// below 64, so (byte | 0x80) - e borrows from no neighbour and keeps its top
+// bit unless the byte is an offset below e
+__device__ __forceinline__ uint32_t msb_below(uint32_t x, uint32_t e) {
+  return ~((x | 0x80808080u) - e * 0x01010101u) & 0x80808080u;
 }
+
+// the axes of an entry that cross before offset e, as an 8-bit mask
+__device__ __forceinline__ uint32_t bytes_below(uint64_t c8, uint32_t e) {
+  return byte_lsbs(msb_below((uint32_t)c8, e) >> 7) | (byte_lsbs(msb_below((uint32_t)(c8 >> 32), e) >> 7) << 4);
+}
+
+// a 4-bit mask as bytes: 0xFF where the bit is set
+__device__ __forceinline__ uint32_t bytes_of(uint32_t m) { return ((m & 0xFu) * 0x00204081u & 0x01010101u) * 0xFFu; }
+
+// 16 bytes of global memory into shared memory, asynchronously, through L2
+// only (a lazy table's rows may have been written by another SM)
+__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // One warp per replica; replicas come from a work list of (simulation,
 // replica) items that every warp pulls from.  There is no CTA barrier: the
 // warp's counters stay in registers, appends to the burning list are placed
 // by ballot + popc, and phases are ordered with __syncwarp.  Per replica: an
-// Available plane (burnable, not harvested, not yet ignited -- an ignition is
-// one atomicAnd, whose old value also picks the single winner) and a Burned
-// plane; with WIN their window around the ignition cell and the burning-list
-// arrays sit in shared memory.  The scar plane (burnable and no longer
-// Available) is written at the end.
+// Available plane (burnable, not harvested, not yet ignited); with WIN its
+// window around the ignition cell and the burning-list arrays sit in shared
+// memory.  The scar plane (burnable and no longer Available) is written at
+// the end.
 //
-// Each hour the burning cells' crossings are kept in a calendar: one linked
-// list of list entries per crossing offset (an entry sits in the list of its
-// earliest crossing) and a 64-bit mask of the offsets whose lists are not
-// empty.  The next fire period to visit is the mask's lowest bit, and a
-// visited period walks only the entries that cross in it.  Work is laid out
-// one lane per cell, the 8 axes of a cell as independent chains in its lane:
-// at the hour boundary (every listed cell) and for the cells ignited in a
-// visited period.
+// Within an hour every axis crosses at a known offset.  The warp advances by
+// windows of consecutive periods [o1, E): no cell that ignites in a window
+// sends before the window's end, so all its crossings are known at its start
+// and are handled at once.  o1 is the lowest bit of a 64-bit calendar mask of
+// the offsets at which some entry crosses; E is found as the window is worked
+// out:
+//   A1  the entries whose earliest crossing lies in [o1, o1 + width), by a
+//       scan of one byte per entry, four to a word, 32 words at a time;
+//   A2  their crossings in the window towards Available cells, one per lane,
+//   A3  ranked by offset; a cell reached several times ignites at the first;
+//   C1  lane i takes the i-th cell to ignite: table row into shared memory
+//       (asynchronously), perturbation;
+//   C2  four cells at a time, lane k of each 8-lane group owning axis k: the
+//       offsets at which the new cells send, progress to the end of the hour;
+//   C3  E = the earliest of these offsets (at most o1 + width); the cells that
+//       ignite before E are taken and listed (the others stay Available and
+//       their crossings open); cells with no Available neighbour left burn
+//       out at the last ignition next to them;
+//   C4  the crossings before E are closed.
+// Every window is at least one period long (a cell sends after the period in
+// which it ignites).  width follows what the last windows reached.  One period
+// at a time a replica of the 512 x 512 landscape issued about 980 instructions
+// in each of its 1,090 visited periods, most of them in passes that few lanes
+// had work for.
 template <int WPC, bool WIN, bool LAZY, bool PROF>
 __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
-  // list links: 16 bits in shared memory (capacities there stay far below 2^16)
-  using Link = typename std::conditional<WIN, uint16_t, int32_t>::type;
-  constexpr int32_t kNil = -1;
   extern __shared__ __align__(16) uint32_t s_dyn[];
   __shared__ SimJob s_job[WPC];
   constexpr uint32_t FULL = 0xffffffffu;
@@ -636,34 +572,35 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   // compact the list within an hour once it holds more than this many entries
   const int32_t compact_at = (A.compact_at > 0 && A.compact_at < cap) ? A.compact_at : cap - cap / 4;
   const uint32_t wait_limit = A.wait_limit ? A.wait_limit : kChunkSpinLimit;
-  uint32_t *my = s_dyn + (size_t)wib * A.smem_warp_words;   // [Available win][Burned win][lists]
+  uint32_t *my = s_dyn + (size_t)wib * A.smem_warp_words;   // [Available window][lists]
   uint32_t *erc;     // row << 16 | col
   uint8_t *ecofs;    // 8 crossing-offset bytes per entry
-  Link *elink;       // next entry in the same calendar list
+  uint8_t *enx;      // the entry's earliest crossing (the least of its 8 bytes)
   Planes<WIN> pl;
   pl.gav = A.avail_scratch + slot * (size_t)A.pw_max;
   pl.gbr = A.brn_scratch + slot * (size_t)A.pw_max;
   if constexpr (WIN) {
     pl.sav = my;
-    pl.sbr = my + kWinRows * kWinWords;
-    uint32_t *ls = my + 2 * kWinRows * kWinWords;
-    erc = ls;
-    ecofs = reinterpret_cast<uint8_t *>(ls + cap);
-    elink = reinterpret_cast<Link *>(ls + 3 * (size_t)cap);
+    uint32_t *ls = my + kWinRows * kWinWords;
+    ecofs = reinterpret_cast<uint8_t *>(ls);
+    erc = ls + 2 * (size_t)cap;
+    enx = reinterpret_cast<uint8_t *>(ls + 3 * (size_t)cap);
   } else {
-    pl.sav = pl.sbr = nullptr;
+    pl.sav = nullptr;
     erc = reinterpret_cast<uint32_t *>(A.ent_cell) + slot * cap;
     ecofs = A.ent_cofs + slot * (size_t)cap * 8;
-    elink = reinterpret_cast<Link *>(A.ent_link) + slot * cap;
+    enx = A.ent_next + slot * (size_t)((cap + 3) & ~3);
   }
   int64_t *eP = A.ent_P + slot * (size_t)cap * 8;
-  __shared__ int32_t s_hits[WPC][32];                  // one round of crossing entries
-  __shared__ int32_t s_head[WPC][64];                  // calendar: first entry per offset
+  __shared__ __align__(16) int64_t s_rows[WPC][32 * 8];   // the new cells' table rows
+  __shared__ uint32_t s_buf[WPC][32];                     // a window's entries, crossings, burn-outs
+  __shared__ uint8_t s_off[WPC][32];                      // the new cells' offsets
   __shared__ uint32_t s_dbits[WPC][LAZY ? kWinRows * kWinWords / 32 : 1];   // chunks known done this hour
   __shared__ int32_t s_claim[WPC][LAZY ? 32 : 1];
   __shared__ long long s_prof[WPC][PROF ? kProfCounters : 1];
-  int32_t *hitbuf = s_hits[wib];
-  int32_t *head = s_head[wib];
+  int64_t *rowbuf = s_rows[wib];
+  uint32_t *buf = s_buf[wib];
+  uint8_t *obuf = s_off[wib];
   uint32_t *dbits = s_dbits[wib];
   int32_t *claim = s_claim[wib];
   SimJob &J = s_job[wib];
@@ -706,11 +643,16 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     const bool lazy = LAZY && J.chunk_state != nullptr;
     const double delta = J.delta;
     const bool use_delta = delta > 0.0;   // A5 (i) burn-out on
+    // the longest window (with A5 (i) a cell may stop before its neighbours
+    // are gone, so burn-outs are settled period by period)
+    const int32_t width_max = use_delta ? 1 : 32;
+    int32_t width = use_delta ? 1 : 4;
     const uint64_t seed = J.seed;
     const float sigma = J.sigma;
     const uint32_t *burnable = J.burnable;
     int32_t *istep = J.ign_step ? J.ign_step + (size_t)r * n : nullptr;
     const int64_t dk = (k & 1) ? J.d_diag : J.d_orth;   // this lane's axis length
+    const int len_shift = max(0, 33 - __clzll(J.d_diag));   // lengths >> len_shift fit 31 bits
     const int32_t ic = J.ign_cell[r];
     // an ignition cell outside the grid or not burnable (possible only for
     // ignition cells a caller passes in): status 3, nothing else is written
@@ -721,9 +663,10 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       continue;
     }
     const int32_t ir = ic / cols, icc = ic - ir * cols;
-    // window of the done-chunk bitmap, centred on the ignition cell like the planes'
+    // window of the done-chunk bitmap, centred on the ignition cell like the plane's
     const int32_t dr0 = min(max(ir - kWinRows / 2, 0), max(rows - kWinRows, 0));
     const int32_t dw0 = min(max((icc >> 5) - kWinWords / 2, 0), max(wpr - kWinWords, 0));
+    pl.rows = rows;
     pl.wpr = wpr;
     bool need_global = true;
     if constexpr (WIN) {   // window centred on the ignition cell, clamped to the grid
@@ -732,26 +675,18 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       need_global = rows > kWinRows || wpr > kWinWords;
       for (int32_t i = lane; i < kWinRows * kWinWords; i += 32) {
         const int32_t rr = pl.r0 + i / kWinWords, ww = pl.w0 + i % kWinWords;
-        const uint32_t b = (rr < rows && ww < wpr) ? __ldg(&burnable[rr * wpr + ww]) : 0u;
-        pl.sav[i] = b;
-        pl.sbr[i] = ~b;   // cells that never burn count as Burned already
+        pl.sav[i] = (rr < rows && ww < wpr) ? __ldg(&burnable[rr * wpr + ww]) : 0u;
       }
     }
     if (need_global)
-      for (int32_t i = lane; i < pw; i += 32) {
-        const uint32_t b = __ldg(&burnable[i]);
-        pl.gav[i] = b;
-        pl.gbr[i] = ~b;
-      }
+      for (int32_t i = lane; i < pw; i += 32) pl.gav[i] = __ldg(&burnable[i]);
+    if (use_delta)
+      for (int32_t i = lane; i < pw; i += 32) pl.gbr[i] = 0u;
     __syncwarp();
 
     // per-replica profile (J.prof, off unless the caller asked for it; the
-    // layout of c2f_get_replica_profile): cycles in all, at hour boundaries,
-    // finding + sending crossings and receiving (A), new-cell set-up (C);
-    // visited periods, crossing entries, new cells, longest list; cycles of
-    // (A) spent walking the period's calendar list, compactions within an
-    // hour, rounds of crossing entries, new-cell passes (32 cells each)
-    // (kept in shared memory, lane 0 only, so that they cost no registers)
+    // layout of c2f_get_replica_profile), kept in shared memory by lane 0 so
+    // that it costs no registers
     const bool prof = PROF && J.prof != nullptr;   // compiled out of the production kernels
     long long pc_t = 0;
     long long *pq = s_prof[wib];
@@ -761,23 +696,27 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       pq[0] = clock64();
     }
 
-    // Step 1 of Alg. 1: the ignition cell burns from period 0
+    // Step 1 of Alg. 1: the ignition cell burns from period 0.  Work: a cell
+    // counts in the periods after its ignition up to its burn-out (or the
+    // end), so W = sum of burn-out periods - ignition periods, less the
+    // dormant hours.
     int32_t live = 1, nign = 1, cnt = 1, status = 0;
-    long long W = 0, s_done = 0;
+    long long W = 0;
     {
       if (lane == 0) {
         pl.take(ir, icc);
         if (istep) istep[ic] = 0;
       }
       __syncwarp();
-      const uint32_t am = pl.avail_mask(rows, cols, ir, icc);
+      uint32_t b[3];
+      pl.template block<1>(ir, icc, b);
+      const uint32_t am = axes_of_rows(b[0], b[1], b[2]);
       if (lane < 8) {
         eP[lane] = 0;
         ecofs[lane] = (uint8_t)(((am >> lane) & 1u) ? kOpen : kNone);
       }
       if (lane == 0) erc[0] = rc_pack(ir, icc);
       if (am == 0) {   // no Available neighbour: Burned at the end of period 1
-        if (lane == 0) pl.burn(ir, icc);
         live = 0;
         W = (H * sph >= 1) ? 1 : 0;
       }
@@ -785,89 +724,84 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     }
 
     // On-demand table rows (lazy tables): before a row of hour h is read, the
-    // chunk holding it must be done.  `slots` bit 0 asks for the cell's own
-    // chunk, bit 1 + k for the chunk of its neighbour on axis k.  A chunk is
-    // looked up in the bitmap of chunks known done this hour, else in
-    // chunk_state: claimed when empty (the warp computes its claims at once,
-    // all lanes on one chunk), waited for when another warp is computing it --
-    // that warp is running and never waits while it holds a claim.
-    auto ensure = [&](int32_t h, bool valid, int32_t cr, int32_t cc, uint32_t slots) {
+    // chunk holding it must be done.  A chunk is looked up in the bitmap of
+    // chunks known done this hour, else in chunk_state: claimed when empty (the
+    // warp computes its claims at once, all lanes on one chunk), waited for
+    // when another warp is computing it -- that warp is running and never
+    // waits while it holds a claim.
+    auto ensure = [&](int32_t h, bool valid, int32_t cr, int32_t cc) {
       if (status != 0) return;   // the replica has stopped: no more claims or waits
-      if (!valid) slots = 0;
-      uint32_t todo = __reduce_or_sync(FULL, slots);
       uint32_t *sth = J.chunk_state + (size_t)h * pw;
-      while (todo) {
-        const int q = __ffs(todo) - 1;
-        todo &= todo - 1;
-        int32_t wr = -1, wc = 0;
-        if ((slots >> q) & 1u) {
-          int32_t nr = cr, nc = cc;
-          if (q > 0) { nr += axis_dr(q - 1); nc += axis_dc(q - 1); }
-          if (nr >= 0 && nr < rows && nc >= 0 && nc < cols) { wr = nr; wc = nc >> 5; }
+      const int32_t wr = cr, wc = cc >> 5;
+      const int32_t w = wr * wpr + wc;
+      const bool inwin = wr >= dr0 && wr < dr0 + kWinRows && wc >= dw0 && wc < dw0 + kWinWords;
+      const int32_t bi = inwin ? (wr - dr0) * kWinWords + (wc - dw0) : 0;
+      bool need = false, mine = false;
+      if (valid && !(inwin && ((dbits[bi >> 5] >> (bi & 31)) & 1u))) {
+        uint32_t st = ld_state(sth + w);
+        if (st == 0u) {
+          st = atomicCAS(sth + w, 0u, 1u);
+          mine = st == 0u;
         }
-        const int32_t w = wr * wpr + wc;
-        const bool inwin = wr >= dr0 && wr < dr0 + kWinRows && wc >= dw0 && wc < dw0 + kWinWords;
-        const int32_t bi = inwin ? (wr - dr0) * kWinWords + (wc - dw0) : 0;
-        bool need = false, mine = false;
-        if (wr >= 0 && !(inwin && ((dbits[bi >> 5] >> (bi & 31)) & 1u))) {
-          uint32_t st = ld_state(sth + w);
-          if (st == 0u) {
-            st = atomicCAS(sth + w, 0u, 1u);
-            mine = st == 0u;
-          }
-          need = !mine && st < 2u;
-          if (st >= 2u && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
-        }
-        const uint32_t mb = __ballot_sync(FULL, mine);
-        if (mine) claim[__popc(mb & lt)] = w;
-        __syncwarp();
-        const int nm = __popc(mb);
-        for (int i = 0; i < nm; ++i) table_chunk(J, h, claim[i]);
-        if (mine && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
-        if (need) {
-          uint32_t polls = 0;
-          bool gave_up = false;
-          while (ld_state(sth + w) < 2u) {
-            if (++polls > wait_limit) { status = 4; gave_up = true; break; }
-            __nanosleep(128);
-          }
-          if (!gave_up && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
-        }
-        __syncwarp();
+        need = !mine && st < 2u;
+        if (st >= 2u && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
       }
+      const uint32_t mb = __ballot_sync(FULL, mine);
+      if (mine) claim[__popc(mb & lt)] = w;
+      __syncwarp();
+      const int nm = __popc(mb);
+      for (int i = 0; i < nm; ++i) table_chunk(J, h, claim[i]);
+      if (mine && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
+      if (need) {
+        uint32_t polls = 0;
+        bool gave_up = false;
+        while (ld_state(sth + w) < 2u) {
+          if (++polls > wait_limit) { status = 4; gave_up = true; break; }
+          __nanosleep(128);
+        }
+        if (!gave_up && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
+      }
+      __syncwarp();
       status = (int32_t)__reduce_max_sync(FULL, (uint32_t)status);   // the warp's worst status
     };
 
-    // calendar: puts entry e into the list of offset nx; returns nx's bit
-    // (0 when the entry has no crossing left this hour)
-    auto push = [&](int32_t e, uint32_t nx) -> uint64_t {
-      if (nx >= (uint32_t)sph) return 0ull;
-      elink[e] = (Link)atom_exch_shared(&head[nx], e);
-      return 1ull << nx;
-    };
+    // the calendar bit of offset nx (0 when it is not a crossing of this hour)
+    auto cal_bit = [&](uint32_t nx) -> uint64_t { return nx < (uint32_t)sph ? 1ull << nx : 0ull; };
     auto cal_or = [&](uint64_t bits) -> uint64_t {   // OR of the lanes' calendar bits
       return ((uint64_t)__reduce_or_sync(FULL, (uint32_t)(bits >> 32)) << 32) |
              (uint64_t)__reduce_or_sync(FULL, (uint32_t)bits);
     };
+    // the scan of A1 reads enx by words: the bytes that share the list's last
+    // word with it hold no crossing
+    auto end_list = [&](int32_t count) {
+      if ((count & 3) != 0 && lane < 4 - (count & 3)) enx[count + lane] = kNone;
+    };
 
-    // drop Burned cells and cells with no open axis from the burning list
-    // (order kept) when it nears its capacity within an hour, and rebuild the
-    // calendar lists of the offsets from o on; returns the new calendar mask
-    auto compact = [&](int32_t &count, uint32_t o) -> uint64_t {
-      for (int32_t i = lane; i < 64; i += 32) head[i] = kNil;
-      __syncwarp();
+    // drop burned-out cells and cells with no open axis from the burning list
+    // (order kept) when it nears its capacity within an hour; the calendar
+    // keeps its bits (an offset whose entries are gone is an empty window)
+    auto compact = [&](int32_t &count) {
       int32_t out = 0;
-      uint64_t cal = 0;
       for (int32_t b0 = 0; b0 < count; b0 += 32) {
         const int32_t e = b0 + lane;
         bool keep = false;
         uint32_t rc = 0;
         uint64_t c8 = ~0ull;
+        uint8_t nx = 0;
         int64_t P[8];
         if (e < count) {
           rc = erc[e];
           c8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8);
-          keep = open_axes(c8) != 0 && !pl.burned((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu));
+          nx = enx[e];
+          const uint32_t m = open_axes(c8);
+          const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
+          if (use_delta) {
+            keep = m != 0u && !pl.burned(cr, cc);
+          } else if (m != 0u) {
+            uint32_t b[3];
+            pl.template block<1>(cr, cc, b);
+            keep = (m & axes_of_rows(b[0], b[1], b[2])) != 0u;
+          }
           if (keep) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) P[q] = eP[(size_t)e * 8 + q];
@@ -876,27 +810,25 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         const uint32_t bal = __ballot_sync(FULL, keep);
         const int32_t pos = out + __popc(bal & lt);
         __syncwarp();
-        uint64_t bit = 0;
         if (keep) {
           erc[pos] = rc;
           *reinterpret_cast<uint64_t *>(ecofs + (size_t)pos * 8) = c8;
+          enx[pos] = nx;
 #pragma unroll
           for (int q = 0; q < 8; ++q) eP[(size_t)pos * 8 + q] = P[q];
-          const uint32_t nx = min_byte8(c8);
-          if (nx >= o) bit = push(pos, nx);
         }
-        cal |= cal_or(bit);
         out += __popc(bal);
         __syncwarp();
       }
       count = out;
-      return cal;
+      end_list(count);
+      __syncwarp();
     };
 
     for (int32_t h = 0; h < H && live > 0 && status == 0; ++h) {
-      const int32_t s0 = h * sph + 1, L = s0 + sph - 1;
+      const int32_t s0 = h * sph + 1;   // the hour's first period
       if (h % 24 >= bhours) {   // a dormant hour: nothing moves, no work is counted
-        s_done = L;
+        W -= (long long)live * sph;
         continue;
       }
       const int64_t *baseh = J.base + (size_t)h * n * 8;
@@ -904,33 +836,37 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       // receive tests can be skipped when the threshold is 0 and every HROS of
       // the hour is positive (then HROS * f > 0), or when the threshold is < 0
       const bool gate_free = J.recv_gate <= 1 || (J.recv_gate == 2 && J.hour && J.hour[h].pos);
-      int32_t burned = 0;   // cells Burned at the end of the period being visited
+      int32_t dying = 0;   // cells Burned at the end of the hour's first period (A5 (i))
       if (lazy) {
         for (int32_t i = lane; i < kWinRows * kWinWords / 32; i += 32) dbits[i] = 0u;
+        __syncwarp();
       }
-      for (int32_t i = lane; i < 64; i += 32) head[i] = kNil;
-      __syncwarp();
-      uint64_t cal = 0;   // offsets of this hour whose calendar list is not empty
+      uint64_t cal = 0;   // offsets of this hour at which some entry crosses
 
       if (prof && lane == 0) pc_t = clock64();
       // ---- hour boundary, one lane per listed cell, 32 cells at a time:
-      // (i) drop Burned cells and cells with no open axis (order kept);
+      // (i) drop burned-out cells and cells with no open axis (order kept);
       // (ii) the cell's perturbation for this hour; (iii) on every open axis,
       // the crossing period of this hour, or the progress carried to the next;
-      // (iv) the cell into the calendar list of its first crossing.
+      // (iv) the offset of its first crossing.
       {
         int32_t out = 0;
         for (int32_t b0 = 0; b0 < cnt; b0 += 32) {
           const int32_t e = b0 + lane;
           bool keep = false;
-          uint32_t rc = 0u, m = 0u;
+          uint32_t rc = 0u, am = 0u;   // am: open axes toward Available cells
           if (e < cnt) {
             rc = erc[e];
-            m = open_axes(*reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8));
-            keep = m != 0u && !pl.burned((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu));
+            const uint32_t m = open_axes(*reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8));
+            const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
+            uint32_t b[3];
+            pl.template block<1>(cr, cc, b);
+            am = m & axes_of_rows(b[0], b[1], b[2]);
+            // with A5 (i) a cell with no way left may still die before its neighbours are gone
+            keep = use_delta ? m != 0u && (b[0] | b[1] | b[2]) != 0u && !pl.burned(cr, cc) : am != 0u;
           }
           const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
-          if (lazy) ensure(h, keep, cr, cc, 1u);   // this hour's row of the cell
+          if (lazy) ensure(h, keep, cr, cc);   // this hour's row of the cell
           const int64_t cell = (int64_t)cr * cols + cc;
           int64_t P[8], bk[8];
           if (keep) {   // progress and rate row: 64 bytes each, four 16-byte loads
@@ -945,6 +881,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
             // the cell's row of the next hour into L2, for the next boundary
             if (!LAZY && h + 1 < H) prefetch_l2(baseh + n * 8 + cell * 8);
           } else {
+            am = 0u;
 #pragma unroll
             for (int q = 0; q < 8; ++q) P[q] = bk[q] = 0;
           }
@@ -954,7 +891,6 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           // first period of the hour and is Burned after it
           const bool dies = keep && use_delta && below_delta(hrosh, cell, f, delta);
           uint64_t c8 = ~0ull;   // crossing-offset bytes
-          const uint32_t am = keep ? (m & pl.avail_mask(rows, cols, cr, cc)) : 0u;   // open axes toward Available cells
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             uint32_t cof = kNone;
@@ -963,7 +899,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
               const int64_t inc = apply_noise(bk[q], F, dq);
               const int64_t rem = dq - P[q];
               if (inc > 0 && inc * sph >= rem) {
-                cof = (uint32_t)(ceil_div_small(rem, inc) - 1);
+                cof = (uint32_t)(ceil_div_small(rem, inc, len_shift) - 1);
               } else {
                 P[q] += inc * sph;
                 cof = kOpen;
@@ -972,203 +908,339 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
             }
             c8 = (c8 & ~(0xFFull << (8 * q))) | ((uint64_t)cof << (8 * q));
           }
-          const bool dying = dies && pl.burn(cr, cc);
+          const bool burns = dies && pl.burn(cr, cc);
           const uint32_t bal = __ballot_sync(FULL, keep);
           const int32_t pos = out + __popc(bal & lt);
           __syncwarp();   // every lane has read its entry before any slot is rewritten
           uint64_t bit = 0;
           if (keep) {
+            const uint32_t nx = min_byte8(c8);
             erc[pos] = rc;
             *reinterpret_cast<uint64_t *>(ecofs + (size_t)pos * 8) = c8;
+            enx[pos] = (uint8_t)nx;
             longlong2 *pp = reinterpret_cast<longlong2 *>(eP + (size_t)pos * 8);
 #pragma unroll
             for (int j = 0; j < 4; ++j) pp[j] = make_longlong2(P[2 * j], P[2 * j + 1]);
-            bit = push(pos, min_byte8(c8));
+            bit = cal_bit(nx);
           }
           cal |= cal_or(bit);
           out += __popc(bal);
-          burned += __popc(__ballot_sync(FULL, dying));
+          if (use_delta) dying += __popc(__ballot_sync(FULL, burns));
           __syncwarp();
         }
         cnt = out;
+        end_list(cnt);
+        __syncwarp();
       }
       if (prof && lane == 0) pq[1] += clock64() - pc_t;
       if (status) break;
-      // cells that die this hour (A5 (i)) are Burned at the end of its first
-      // period: that period is visited even if no axis crosses in it
-      if (burned) cal |= 1ull;
+      live -= dying;
+      W += (long long)dying * s0;
 
-      // ---- periods of this hour at which some axis reaches a centre
+      // ---- the periods of this hour at which some axis reaches a centre
       while (cal != 0ull) {
-        const uint32_t o = (uint32_t)(__ffsll((long long)cal) - 1);
-        const int32_t s = s0 + (int32_t)o;
-        W += (long long)live * (long long)(s - s_done);
-        s_done = s;
-        if (prof && lane == 0) { pc_t = clock64(); pq[4] += 1; pq[7] = max(pq[7], (long long)cnt); }
+        const int32_t o1 = __ffsll((long long)cal) - 1;
+        if (prof && lane == 0) { pc_t = clock64(); pq[7] = max(pq[7], (long long)cnt); }
         if (cnt > compact_at) {   // keep room for new cells
-          cal = compact(cnt, o);
+          compact(cnt);
           if (prof && lane == 0) pq[9] += 1;
         }
-        cal &= ~(1ull << o);
-        int32_t nnew = cnt;
-        bool ovf = false;
-        // (A) send and receive: the entries of offset o's calendar list, 32 at
-        // a time (lane 0 walks the list); each lane takes one entry: every
-        // axis crossing at o is handled in turn (target tested, ignited,
-        // appended by ballot + popc), then the entry goes into the list of its
-        // next crossing
-        int32_t cur = head[o];
-        int32_t walked = 0;   // a list holds each entry at most once: never more than cnt
-        while (cur != kNil) {
-          long long pw0 = 0;
-          if (prof && lane == 0) pw0 = clock64();
-          int32_t take_n = 0;
-          if (lane == 0) {
-            while (cur != kNil && take_n < 32) {
-              hitbuf[take_n++] = cur;
-              cur = elink[cur];
-              if (cur == (int32_t)(Link)kNil) cur = kNil;
-            }
-          }
-          take_n = __shfl_sync(FULL, take_n, 0);
-          cur = __shfl_sync(FULL, cur, 0);
-          __syncwarp();
-          walked += take_n;
-          if (walked > cnt) { status = 2; break; }   // cannot happen; a broken list stops here
-          if (prof && lane == 0) { pq[8] += clock64() - pw0; pq[5] += take_n; pq[10] += 1; }
-          const int32_t ent = lane < take_n ? hitbuf[lane] : -1;
-          uint64_t cof8 = ~0ull;
-          uint32_t rc = 0;
-          if (ent >= 0) {
-            cof8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)ent * 8);
-            rc = erc[ent];
-          }
-          const uint32_t cm = ent >= 0 ? axes_at(cof8, o) : 0u;   // axes crossing at o
-          const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
-          if (lazy && !gate_free) ensure(h, ent >= 0, cr, cc, cm << 1);   // receivers' HROS
-          uint32_t todo = cm;
-          const int rounds = (int)__reduce_max_sync(FULL, (uint32_t)__popc(cm));
-          for (int it2 = 0; it2 < rounds; ++it2) {
-            bool won = false;
-            uint32_t wrc = 0;
-            int64_t jc = 0;
-            if (todo) {
-              const int q = __ffs(todo) - 1;
-              todo &= todo - 1;
-              const int32_t nr = cr + axis_dr(q), nc = cc + axis_dc(q);
-              jc = (int64_t)nr * cols + nc;
-              wrc = rc_pack(nr, nc);
-              if (gate_free) {
-                won = pl.take(nr, nc);   // taken iff it was Available; one atomic decides
-              } else if (pl.avail(nr, nc) && receive_ok(J, r, jc, h, n)) {   // else consumed
-                won = pl.take(nr, nc);
-              }
-            }
-            const uint32_t wins = __ballot_sync(FULL, won);
-            if (won) {
-              const int32_t idx = nnew + __popc(wins & lt);
-              if (idx < cap) erc[idx] = wrc; else ovf = true;
-              if (istep) istep[jc] = s;
-              // the new cell's table row, read when it is set up: into L1 when
-              // the table is complete (read-only here), else into L2
-              if (LAZY) prefetch_l2(baseh + jc * 8);
-              else prefetch_row_l1(baseh + jc * 8);
-            }
-            nnew += __popc(wins);
-          }
-          uint64_t bit = 0;
-          if (ent >= 0) {   // the axes that crossed close; the entry moves to its next crossing
-            uint64_t nc8 = cof8;
+        const int32_t Ew = min(o1 + width, sph);   // the window is [o1, Ew), shortened below
+        // (A1) the entries that cross in the window, up to 32
+        int32_t got = 0;
+        bool full = false;
+        for (int32_t g0 = 0; g0 < cnt && !full; g0 += 1024) {
+          uint32_t w = 0;   // bit 8 b + 7 - j: byte b of this lane's j-th word crosses
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              if ((cm >> q) & 1u) nc8 |= 0xFFull << (8 * q);
-            *reinterpret_cast<uint64_t *>(ecofs + (size_t)ent * 8) = nc8;
-            bit = push(ent, min_byte8(nc8));
+          for (int j = 0; j < 8; ++j) {
+            const int32_t e0 = g0 + (j * 32 + lane) * 4;
+            if (g0 + j * 128 >= cnt) break;
+            if (e0 < cnt) w |= msb_below(*reinterpret_cast<const uint32_t *>(enx + e0), (uint32_t)Ew) >> j;
           }
-          cal |= cal_or(bit);
-          __syncwarp();
+          for (;;) {
+            const uint32_t bal = __ballot_sync(FULL, w != 0u);
+            if (bal == 0u) break;
+            const int32_t pos = got + __popc(bal & lt);
+            if (w && pos < 32) {
+              const int32_t b = 31 - __clz((int)w);
+              w ^= 1u << b;
+              buf[pos] = (uint32_t)(g0 + ((7 - (b & 7)) * 32 + lane) * 4 + (b >> 3));
+            }
+            got += __popc(bal);
+            if (got > 32) { full = true; break; }
+          }
         }
+        __syncwarp();
+        if (full && width > 1) { width >>= 1; continue; }   // more than 32: a shorter window
+        got = min(got, 32);
+        if (prof && lane == 0) pq[8] += clock64() - pc_t;
+        if (got == 0) { cal &= ~(1ull << o1); continue; }   // its entries were dropped by a compaction
+        const int32_t ent = lane < got ? (int32_t)buf[lane] : -1;
+        // (A2) the axes that cross in the window, towards Available cells
+        uint64_t cof8 = ~0ull;
+        uint32_t rc = 0u, cand = 0u;
+        if (ent >= 0) {
+          cof8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)ent * 8);
+          rc = erc[ent];
+          cand = bytes_below(cof8, (uint32_t)Ew);
+        }
+        // every gathered entry closes an axis, or the hour would not end; cannot happen
+        if (__any_sync(FULL, ent >= 0 && cand == 0u)) { status = 2; break; }
+        if (ent >= 0) {
+          uint32_t b[3];
+          pl.template block<1>((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu), b);
+          cand &= axes_of_rows(b[0], b[1], b[2]);
+        }
+        uint32_t left = cand;
+        int32_t np = 0;   // crossings (entry lane | axis << 5 | offset << 8) into buf
+        while (np < 32) {
+          const uint32_t bal = __ballot_sync(FULL, left != 0u);
+          if (bal == 0u) break;
+          const int32_t pos = np + __popc(bal & lt);
+          if (left && pos < 32) {
+            const uint32_t q = (uint32_t)(__ffs(left) - 1);
+            left &= left - 1u;
+            buf[pos] = (uint32_t)lane | (q << 5) |
+                       ((__byte_perm((uint32_t)cof8, (uint32_t)(cof8 >> 32), q) & 0xFFu) << 8);
+          }
+          np += __popc(bal);
+        }
+        const bool more = __any_sync(FULL, left != 0u);   // more than 32 crossings
+        __syncwarp();
+        if (more && width > 1) { width >>= 1; continue; }
+        np = min(np, 32);
+        // (A3) in the order of their offsets (rank by the offset's bits), one crossing per lane
+        uint32_t pr = lane < np ? buf[lane] : 0u;
+        if (width > 1) {
+          const uint32_t v = (pr >> 8) - (uint32_t)o1;
+          uint32_t eq = np >= 32 ? FULL : (1u << np) - 1u;
+          int32_t pos = 0;
+#pragma unroll
+          for (int j = 4; j >= 0; --j) {
+            const uint32_t bal = __ballot_sync(FULL, (v >> j) & 1u);
+            if ((v >> j) & 1u) {
+              pos += __popc(eq & ~bal);
+              eq &= bal;
+            } else {
+              eq &= ~bal;
+            }
+          }
+          pos += __popc(eq & lt);
+          __syncwarp();
+          if (lane < np) buf[pos] = pr;
+          __syncwarp();
+          pr = lane < np ? buf[lane] : 0u;
+        }
+        const uint32_t src = __shfl_sync(FULL, rc, (int)(pr & 31u));
+        const int q = (int)((pr >> 5) & 7u);
+        const int32_t tr = (int32_t)(src >> 16) + axis_dr(q), tc = (int32_t)(src & 0xFFFFu) + axis_dc(q);
+        bool hit = lane < np;
+        if (lazy && !gate_free) {   // the receivers' HROS
+          ensure(h, hit, tr, tc);
+          if (status) break;
+        }
+        if (!gate_free && hit) hit = receive_ok(J, r, (int64_t)tr * cols + tc, h, n);   // else consumed
+        // a cell reached by several crossings ignites at the first of them (row
+        // 65535 does not exist, so the idle lanes' keys are no cell)
+        const uint32_t peers = __match_any_sync(FULL, hit ? rc_pack(tr, tc) : (0xFFFF0000u | (uint32_t)lane));
+        const bool won = hit && (peers & lt) == 0u;
+        const uint32_t wins = __ballot_sync(FULL, won);
+        const int32_t nc = __popc(wins);
+        if (won) {
+          buf[__popc(wins & lt)] = rc_pack(tr, tc);
+          obuf[__popc(wins & lt)] = (uint8_t)(pr >> 8);
+        }
+        __syncwarp();
         if (prof && lane == 0) {
           const long long t1 = clock64();
           pq[2] += t1 - pc_t;
           pc_t = t1;
-          pq[6] += nnew - cnt;
+          pq[10] += 1;
         }
-        if (status) break;
-        if (__any_sync(FULL, ovf)) { status = 1; break; }
-        __syncwarp();
-        // (C) cells ignited in period s, four at a time, lane k of each 8-lane
-        // group owning axis k: open axes, first crossings, progress to the end
-        // of the hour, burn-out tests, and the cell into the calendar
+        if (cnt + nc > cap) { status = 1; break; }
+        // (C1) lane i holds the i-th cell that ignites
+        const bool act = lane < nc;
+        const uint32_t nrc = act ? buf[lane] : 0u, no = act ? obuf[lane] : 0u;
+        const int32_t nr = (int32_t)(nrc >> 16), ncol = (int32_t)(nrc & 0xFFFFu);
+        const int64_t ncell = (int64_t)nr * cols + ncol;
         if (lazy) {   // this hour's rows of the new cells
-          for (int32_t b0 = cnt; b0 < nnew; b0 += 32) {
-            const int32_t e = b0 + lane;
-            const uint32_t rc = e < nnew ? erc[e] : 0u;
-            ensure(h, e < nnew, (int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu), 1u);
-          }
+          ensure(h, act, nr, ncol);
           if (status) break;
         }
-        for (int32_t b0 = cnt; b0 < nnew; b0 += 4) {
-          if (prof && lane == 0) pq[11] += 1;
-          const int32_t e = b0 + grp;
-          const bool act = e < nnew;
-          const uint32_t rc = act ? erc[e] : 0u;
-          const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
-          const int64_t cell = (int64_t)cr * cols + cc;
-          const int32_t nr = cr + axis_dr(k), nc = cc + axis_dc(k);
-          const bool ingrid = act && nr >= 0 && nr < rows && nc >= 0 && nc < cols;
-          // the table load issued early; through L1 (the row was prefetched
-          // there) unless other warps may be writing the table (lazy rows)
-          const int64_t bk = act ? (LAZY ? __ldcg(baseh + cell * 8 + k) : __ldca(baseh + cell * 8 + k)) : 0;
-          const bool open = ingrid && pl.avail(nr, nc);
-          // the perturbation does not depend on the loads above: computed while they are in flight
-          const float f = act ? noise_factor(seed, (uint32_t)r, (uint32_t)cell, (uint32_t)h, sigma) : 1.0f;
-          const bool ignq = ingrid && !open;   // ignited, or never burnable (pre-marked Burned)
-          const uint32_t omask = group_bits(open);
-          uint32_t mask = omask;
-          bool dies = false;
-          if (act && use_delta) {
-            if (below_delta(hrosh, cell, f, delta)) { dies = true; mask = 0; }   // A5 (i)
-          }
-          uint32_t cof = ((mask >> k) & 1u) ? kOpen : kNone;
+        float f = 1.0f;
+        uint32_t nam = 0u;   // its axes towards Available cells | offset << 8
+        bool dies = false;
+        if (act) {
+          const int64_t *row = baseh + ncell * 8;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) copy_async16(rowbuf + lane * 8 + 2 * j, row + 2 * j);
+          uint32_t b[3];
+          pl.template block<1>(nr, ncol, b);
+          nam = axes_of_rows(b[0], b[1], b[2]) | (no << 8);
+          f = noise_factor(seed, (uint32_t)r, (uint32_t)ncell, (uint32_t)h, sigma);
+          if (use_delta && below_delta(hrosh, ncell, f, delta)) { dies = true; nam &= ~0xFFu; }   // A5 (i)
+        }
+        copy_async_wait();
+        __syncwarp();
+        // (C2) four cells at a time, lane k of each 8-lane group owning axis k:
+        // first crossings, progress to the end of the hour
+        for (int32_t b0 = 0; b0 < nc; b0 += 4) {
+          const int32_t i = b0 + grp;
+          const uint32_t oa = __shfl_sync(FULL, nam, i & 31);
+          const float fi = __shfl_sync(FULL, f, i & 31);
+          uint32_t cof = kNone;
           int64_t P = 0;
-          if (act && ((mask >> k) & 1u) && s < L) {
-            const int32_t nmax = L - s;   // periods left in the hour
-            const int64_t inc = apply_noise(bk, noise_fixed(f), dk);
-            if (inc > 0 && inc * nmax >= dk) cof = o + (uint32_t)ceil_div_small(dk, inc);
+          if ((oa >> k) & 1u) {
+            const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // periods left in the hour
+            const int64_t inc = apply_noise(rowbuf[i * 8 + k], noise_fixed(fi), dk);
+            cof = kOpen;
+            if (inc > 0 && inc * nmax >= dk) cof = (uint32_t)(o + ceil_div_small(dk, inc, len_shift));
             else P = inc * nmax;
           }
-          const uint32_t nx = group_min(cof);
-          uint32_t newly = 0;   // cells this lane turned Burned (its own cell, its axis neighbour)
-          uint64_t bit = 0;
-          if (act) {
-            ecofs[(size_t)e * 8 + k] = (uint8_t)cof;
-            eP[(size_t)e * 8 + k] = P;
-            if (k == 0) {
-              bit = push(e, nx);
-              if (omask == 0 || dies)   // this cell: A5 (ii) no Available neighbour, or (i)
-                newly += pl.burn(cr, cc) ? 1u : 0u;
-            }
-            // A5 (ii) for the ignited neighbour on this lane's axis
-            if (ignq && !pl.any_avail_nbr(rows, cols, nr, nc)) newly += pl.burn(nr, nc) ? 1u : 0u;
+          if (i < nc) {
+            ecofs[(size_t)(cnt + i) * 8 + k] = (uint8_t)cof;
+            eP[(size_t)(cnt + i) * 8 + k] = P;
           }
-          cal |= cal_or(bit);
-          burned += (int32_t)__reduce_add_sync(FULL, newly);
         }
         __syncwarp();
-        if (prof && lane == 0) pq[3] += clock64() - pc_t;
-        // every crossing pushed in this period lies after it; a bit at or
-        // before o cannot happen and would revisit a period
-        if (cal & ((2ull << o) - 1ull)) { status = 2; break; }
-        const int32_t added = nnew - cnt;
-        nign += added;
-        live += added - burned;
-        burned = 0;
-        cnt = nnew;
+        // (C3) the window's end, and the cells that ignite before it: taken and listed
+        uint64_t c8 = ~0ull;
+        if (act) c8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)(cnt + lane) * 8);
+        const int32_t E = (int32_t)min((uint32_t)Ew, warp_min(min_byte8(c8)));
+        const bool commit = act && (int32_t)no < E;
+        const int32_t done = __popc(__ballot_sync(FULL, commit));
+        uint64_t bits = 0;      // calendar bits this lane sets
+        uint32_t out = 0;       // cells this lane turned Burned: count << 16 | sum of their offsets
+        if (commit) pl.take(nr, ncol);
+        __syncwarp();
+        uint32_t gone = 0u;     // 3 x 3 positions around the cell whose blocks hold no Available cell
+        if (commit) {
+          uint32_t b[5];
+          pl.template block<2>(nr, ncol, b);
+          const uint32_t am = axes_of_rows((b[1] >> 1) & 7u, (b[2] >> 1) & 7u, (b[3] >> 1) & 7u);
+          c8 |= ((uint64_t)bytes_of(~am >> 4) << 32) | bytes_of(~am);   // the axes that are still open
+          const uint32_t nx = min_byte8(c8);
+          erc[cnt + lane] = nrc;
+          *reinterpret_cast<uint64_t *>(ecofs + (size_t)(cnt + lane) * 8) = c8;
+          enx[cnt + lane] = (uint8_t)nx;
+          if (istep) istep[ncell] = s0 + (int32_t)no;
+          bits = cal_bit(nx);
+          if (dies && pl.burn(nr, ncol)) out = (1u << 16) + no;
+          const uint32_t v0 = b[0] | b[1] | b[2], v1 = b[1] | b[2] | b[3], v2 = b[2] | b[3] | b[4];
+          gone = ~((v0 | (v0 >> 1) | (v0 >> 2)) & 7u | (((v1 | (v1 >> 1) | (v1 >> 2)) & 7u) << 3) |
+                   (((v2 | (v2 >> 1) | (v2 >> 2)) & 7u) << 6)) & 0x1FFu;
+        }
+        // A5 (ii): the ignited cells among them have burned out in this window
+        // (a cell next to an ignition of the window had an Available neighbour
+        // before it), at the last ignition next to them
+        if (__any_sync(FULL, gone != 0u)) {
+          uint32_t fuel9 = 0u;   // burnable cells of the 3 x 3 positions
+          if (gone) {
+            const int32_t wl = (ncol - 1) >> 5, wh = (ncol + 1) >> 5;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const int32_t rr = nr - 1 + d;
+              uint32_t lo = 0u, hi = 0u;
+              if (rr >= 0 && rr < rows) {
+                if (wl >= 0) lo = __ldg(&burnable[rr * wpr + wl]);
+                if (wh < wpr) hi = __ldg(&burnable[rr * wpr + wh]);
+              }
+              fuel9 |= (__funnelshift_r(lo, hi, (uint32_t)(ncol - 1) & 31u) & 7u) << (3 * d);
+            }
+          }
+          gone &= fuel9;
+          // the last cells' first: places counted from the highest lane
+          const uint32_t ng = (uint32_t)__popc(gone);
+          int32_t at = 0, total = 0;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t bal = __ballot_sync(FULL, (ng >> j) & 1u);
+            at += __popc(bal & ~lt & ~(1u << lane)) << j;
+            total += __popc(bal) << j;
+          }
+          for (int32_t t0 = 0; t0 < total; t0 += 32) {
+            while (gone != 0u && at < t0 + 32) {
+              const uint32_t p = (uint32_t)(__ffs(gone) - 1);
+              gone &= gone - 1u;
+              buf[at - t0] = (uint32_t)lane | (p << 5);
+              ++at;
+            }
+            __syncwarp();
+            const bool valid = t0 + lane < total;
+            const uint32_t c = valid ? buf[lane] : 0u;
+            const uint32_t crc = __shfl_sync(FULL, nrc, (int)(c & 31u));
+            const uint32_t co = __shfl_sync(FULL, no, (int)(c & 31u));
+            const int32_t p = (int32_t)(c >> 5), pr3 = (p * 11) >> 5;   // p / 3
+            const int32_t xr = (int32_t)(crc >> 16) + pr3 - 1, xc = (int32_t)(crc & 0xFFFFu) + p - 3 * pr3 - 1;
+            bool first;
+            if (total <= 32) {
+              const uint32_t same = __match_any_sync(FULL, valid ? rc_pack(xr, xc) : (0xFFFF0000u | (uint32_t)lane));
+              first = (same & lt) == 0u;
+            } else {   // no later ignition next to it
+              first = true;
+              for (int32_t j = 0; j < done; ++j) {
+                const uint32_t jrc = __shfl_sync(FULL, nrc, j);
+                if (j > (int32_t)(c & 31u) && abs((int32_t)(jrc >> 16) - xr) <= 1 && abs((int32_t)(jrc & 0xFFFFu) - xc) <= 1)
+                  first = false;
+              }
+            }
+            if (valid && first && (!use_delta || pl.burn(xr, xc))) out += (1u << 16) + co;
+            __syncwarp();
+          }
+        }
+        // (C4) the crossings before E are closed
+        if (!full) cal &= ~((1ull << E) - 1ull);   // E <= 60
+        const uint64_t old8 = cof8;
+        if (ent >= 0) {
+          uint32_t lo = msb_below((uint32_t)cof8, (uint32_t)E), hi = msb_below((uint32_t)(cof8 >> 32), (uint32_t)E);
+          if (more) {   // crossings that found no lane stay open
+            lo &= ~bytes_of(left);
+            hi &= ~bytes_of(left >> 4);
+          }
+          if (lo | hi) {
+            cof8 = ((uint64_t)((uint32_t)(cof8 >> 32) | (hi >> 7) * 0xFFu) << 32) | ((uint32_t)cof8 | (lo >> 7) * 0xFFu);
+            const uint32_t nx = min_byte8(cof8);
+            *reinterpret_cast<uint64_t *>(ecofs + (size_t)ent * 8) = cof8;
+            enx[ent] = (uint8_t)nx;
+            bits |= cal_bit(nx);
+          } else if (more) {
+            bits |= 1ull << o1;
+          }
+        }
+        cal |= cal_or(bits);
+        const uint32_t ob = __reduce_add_sync(FULL, out);
+        const int32_t on = (int32_t)__reduce_add_sync(FULL, commit ? no : 0u);
+        const int32_t burned = (int32_t)(ob >> 16);
+        W += (long long)(burned - done) * s0 + ((int32_t)(ob & 0xFFFFu) - on);
+        if (PROF) {
+          uint64_t seen = 0;   // periods at which a crossing was processed
+          if (prof && cof8 != old8) {
+            for (int j = 0; j < 8; ++j) {
+              const uint32_t u = (uint32_t)(old8 >> (8 * j)) & 0xFFu;
+              if ((int32_t)u < E) seen |= 1ull << u;
+            }
+          }
+          const int32_t ch = __popc(__ballot_sync(FULL, cof8 != old8));
+          seen = cal_or(seen);
+          if (prof && lane == 0) {
+            pq[3] += clock64() - pc_t;
+            if (!full && !more) pq[4] += __popcll(seen);
+            pq[5] += ch;
+            pq[6] += done;
+            pq[11] += (done + 3) / 4;
+          }
+        }
+        nign += done;
+        live += done - burned;
+        cnt += done;
+        end_list(cnt);
+        // the next window: a little longer than what this one reached
+        width = E < Ew ? min(width, E - o1 + 2) : min(2 * width, width_max);
+        __syncwarp();
         if (live == 0) break;
       }
-      if (status == 0) { W += (long long)live * (long long)(L - s_done); s_done = L; }
     }
+    W += (long long)live * (long long)H * sph;
     {   // scar plane: burnable cells that are no longer Available
       uint32_t *dst = J.ign_plane + (size_t)r * pw;
       for (int32_t i = lane; i < pw; i += 32) {

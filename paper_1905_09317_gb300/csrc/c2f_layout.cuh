@@ -112,12 +112,12 @@ struct FrontierArgs {
   unsigned long long *counter;    // work-list cursor (zeroed before the launch)
   int32_t cap;                    // burning-list capacity per slot
   int32_t *ent_cell;              // [slots][cap] cell as row << 16 | col
-  int32_t *ent_link;              // [slots][cap] next entry in the same calendar list (-1 none)
+  uint8_t *ent_next;              // [slots][cap rounded up to 4] the entry's earliest crossing offset
   uint8_t *ent_cofs;              // [slots][cap][8] per-axis crossing offsets this hour
                                   //   (0xFE open axis, no crossing this hour; 0xFF closed)
   int64_t *ent_P;                 // [slots][cap][8] progress at the start of the next hour
   int64_t pw_max;                 // words per bit plane of the largest landscape
-  uint32_t *brn_scratch;          // [slots][pw_max] Burned planes
+  uint32_t *brn_scratch;          // [slots][pw_max] cells burned out by rate (A5 (i)), if that is on
   uint32_t *avail_scratch;        // [slots][pw_max] Available planes (global-plane variant)
   int64_t smem_warp_words;        // 32-bit words of dynamic shared memory per warp
   uint32_t wait_limit;            // polls before a wait for a table chunk gives up; 0 = default
@@ -160,7 +160,7 @@ constexpr int kOrderBuckets = 2 * 16;   // (fuel code, slope > 0); code 0 = not 
 
 constexpr uint8_t kNone = 0xFF;
 constexpr int kProfCounters = 16;   // per-replica frontier profile counters (c2f_get_replica_profile)
-// shared-memory window of the per-replica bit planes: kWinRows x (32 kWinWords) cells
+// shared-memory window of the per-replica Available plane: kWinRows x (32 kWinWords) cells
 constexpr int kWinRows = 256;
 constexpr int kWinWords = 8;
 

@@ -355,11 +355,9 @@ __device__ inline float fcos_turns(float u) {
 #pragma unroll
   for (int n = 4; n >= 1; --n) pc = __fmaf_rn(pc, t2, g_mc.cos_cf[n]);
   const float cs = __fmaf_rn(t2, pc, 1.0f);
-  const int q = ((((int)qf) % 4) + 4) % 4;
-  if (q == 0) return cs;
-  if (q == 1) return -sn;
-  if (q == 2) return -cs;
-  return sn;
+  const int q = (int)qf & 3;   // quadrants 0..3: cs, -sn, -cs, sn
+  const float v = (q & 1) ? sn : cs;
+  return __int_as_float(__float_as_int(v) ^ (((q + 1) & 2) << 30));
 }
 
 // ---------------------------------------------------------------- Philox
@@ -402,16 +400,17 @@ __device__ __forceinline__ uint64_t noise_fixed(float f) {
   return m << ((int)(b >> 23) - 118);   // 2^(e - 127 - 23 + 32), e >= 118 for f >= 2^-9
 }
 
-// per-period increment (base * F + 2^31) >> 32, capped at the axis length
+// per-period increment (base * F + 2^31) >> 32, capped at the axis length dk <
+// 2^53, for 2^23 <= F < 2^41, from the 32-bit halves: with base = b1 2^32 + b0
+// and F = f1 2^32 + f0 it is b1 f1 2^32 + b1 f0 + b0 f1 + ((b0 f0 + 2^31) >> 32).
+// base >= 2^62 or b1 f1 >= 2^21 alone exceeds any dk; otherwise the sum stays
+// below 2^63
 __device__ __forceinline__ int64_t apply_noise(int64_t base, uint64_t F, int64_t dk) {
-  const uint64_t b = (uint64_t)base;
-  uint64_t lo = b * F;
-  uint64_t hi = __umul64hi(b, F);
-  const uint64_t lo2 = lo + 0x80000000ULL;
-  hi += (lo2 < lo) ? 1ULL : 0ULL;
-  // inc = (hi:lo2) >> 32
-  if (hi >> 32) return dk;
-  const uint64_t inc = (hi << 32) | (lo2 >> 32);
+  const uint32_t b0 = (uint32_t)base, b1 = (uint32_t)((uint64_t)base >> 32);
+  const uint32_t f0 = (uint32_t)F, f1 = (uint32_t)(F >> 32);
+  const uint64_t top = (uint64_t)b1 * f1;
+  if ((top >> 21) | (b1 >> 30)) return dk;
+  const uint64_t inc = (top << 32) + (uint64_t)b1 * f0 + (uint64_t)b0 * f1 + (((uint64_t)b0 * f0 + 0x80000000ull) >> 32);
   return inc > (uint64_t)dk ? dk : (int64_t)inc;
 }
 

@@ -179,10 +179,10 @@ struct Sim {
 };
 
 struct Scratch {
-  DevBuf ent_cell, ent_link, ent_cofs, ent_P, counter, brn, avail;
+  DevBuf ent_cell, ent_next, ent_cofs, ent_P, counter, brn, avail;
   int64_t slots = 0, cap = 0, brn_words = 0, avail_words = 0;
   void reset() {
-    ent_cell.reset(); ent_link.reset(); ent_cofs.reset(); ent_P.reset();
+    ent_cell.reset(); ent_next.reset(); ent_cofs.reset(); ent_P.reset();
     counter.reset(); brn.reset(); avail.reset();
     slots = cap = brn_words = avail_words = 0;
   }
@@ -547,6 +547,7 @@ std::shared_ptr<Sim> find_sim(c2f_ctx *ctx, int32_t id) {
 }
 
 constexpr int64_t kCoRunSmem = 12 * 1024;
+constexpr int64_t kEntryBytes = 13;   // a burning-list entry in shared memory: cell, 8 crossing offsets, the first
 
 int64_t default_cap(const c2f_ctx *ctx, const Landscape &L) {
   if (ctx->cap_override > 0) return std::min<int64_t>(L.n, ctx->cap_override);
@@ -564,7 +565,7 @@ int ensure_scratch_once(c2f_ctx *ctx, Scratch &S, cudaStream_t st, int64_t slots
     cap = std::max(cap, S.cap);
     const size_t sc = (size_t)slots * cap;
     if ((rc = dalloc_on(ctx, S.ent_cell, sc * 4, st))) return rc;
-    if ((rc = dalloc_on(ctx, S.ent_link, sc * 4, st))) return rc;
+    if ((rc = dalloc_on(ctx, S.ent_next, (size_t)slots * ((cap + 3) & ~int64_t(3)), st))) return rc;
     if ((rc = dalloc_on(ctx, S.ent_cofs, sc * 8, st))) return rc;
     if ((rc = dalloc_on(ctx, S.ent_P, sc * 64, st))) return rc;
     S.slots = slots;
@@ -697,20 +698,20 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
     const int64_t warps_per_sm =
         attempt == 0 ? (ctx->warps_per_sm > 0 ? (int64_t)ctx->warps_per_sm : std::min<int64_t>(want, 8))
                      : std::min<int64_t>(want, 2);
-    // per CTA: 1 KB reserved by the system and about 1.3 KB of static shared
-    // memory per warp; with the default sizing, kCoRunSmem per SM is left for
+    // per CTA: 1 KB reserved by the system and about 3 KB of static shared
+    // memory per warp (2 KB of them the new cells' table rows); with the default sizing, kCoRunSmem per SM is left for
     // kernels that run beside the frontier (the next step's or request's table
     // build, burn counts), whose CTAs could not be placed on a full SM
     const int64_t reserve = (attempt == 0 && ctx->warps_per_sm == 0) ? kCoRunSmem : 0;
     const int64_t per_warp = ((int64_t)ctx->smem_per_sm - reserve - (1024 * warps_per_sm) / wpc -
-                              1300 * warps_per_sm) / warps_per_sm;
-    const int64_t room = (per_warp - 2 * (int64_t)kWinRows * kWinWords * 4 - 512) / 14;
+                              3000 * warps_per_sm) / warps_per_sm;
+    const int64_t room = (per_warp - (int64_t)kWinRows * kWinWords * 4 - 512) / kEntryBytes;
     win_cap = std::min<int64_t>(cap, std::max<int64_t>(256, room & ~int64_t(63)));
     if (attempt > 0) win_cap = std::max<int64_t>(256, room & ~int64_t(63));
-    win_cap = std::min<int64_t>(win_cap, 65532);   // shared-memory lists link entries with 16 bits
   }
-  const int64_t budget = (int64_t)ctx->smem_optin - 2048;
-  const int64_t win_words = 2 * (int64_t)kWinRows * kWinWords + win_cap * 7 / 2;
+  const int64_t budget = (int64_t)ctx->smem_optin - 3072 * wpc;
+  // (a warp's share is rounded up to 16 bytes: the next warp's lists are read 8 bytes at a time)
+  const int64_t win_words = ((int64_t)kWinRows * kWinWords + win_cap * kEntryBytes / 4 + 3) & ~int64_t(3);
   // shared-memory lists only when they hold at least 40 % of the default
   // capacity: smaller ones overflow on large fires and those replicas run twice
   const bool use_win = ctx->window_smem && win_words * 4 * wpc <= budget &&
@@ -747,7 +748,7 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
   A.counter = S.counter.as<unsigned long long>();
   A.cap = (int32_t)cap;
   A.ent_cell = S.ent_cell.as<int32_t>();
-  A.ent_link = S.ent_link.as<int32_t>();
+  A.ent_next = S.ent_next.as<uint8_t>();
   A.ent_cofs = S.ent_cofs.as<uint8_t>();
   A.ent_P = S.ent_P.as<int64_t>();
   A.pw_max = F.pw_max;
