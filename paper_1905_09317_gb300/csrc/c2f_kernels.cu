@@ -330,18 +330,22 @@ __device__ __forceinline__ uint32_t min_byte8(uint64_t v) {
   return min(m & 0xFFFFu, m >> 16);
 }
 
-// smallest n >= 1 with n * inc >= rem, for callers that know 0 < inc, 0 < rem
-// and 64 * inc >= rem (a crossing within the hour: at most 60 periods), with
-// rem and inc both below 2^(31 + shift).  A binary32 estimate of the quotient
-// from the top bits, never more than its ceiling (inc is rounded up), then one
-// exact int64 step; the estimate falls short by two or more only when the top
-// bits of inc are few, i.e. for a last few units of a nearly finished axis.
-__device__ __forceinline__ int32_t ceil_div_small(int64_t rem, int64_t inc, int shift) {
+// The number of periods n <= nmax after which an axis with rem > 0 to go
+// reaches its neighbour's centre at inc a period (the smallest n >= 1 with
+// n * inc >= rem), or 0 if it takes more than nmax <= 60; rem and inc are below
+// 2^(31 + shift).  A binary32 estimate of the quotient from the top bits, never
+// more than its ceiling (inc is rounded up), then one exact int64 step; the
+// estimate falls short by two or more only when inc has few top bits, i.e. for
+// the last few units of a nearly finished axis.
+__device__ __forceinline__ int32_t periods_to_cross(int64_t rem, int64_t inc, int32_t nmax, int shift) {
+  const bool in_time = inc > 0 && inc * nmax >= rem;
   const float a = (float)(uint32_t)((uint64_t)rem >> shift), b = (float)((uint32_t)((uint64_t)inc >> shift) + 1u);
-  int32_t n = (int32_t)__fdividef(a, b);
-  int64_t left = rem - (int64_t)n * inc;
-  while (left > 0) { ++n; left -= inc; }
-  return n;
+  int32_t n = in_time ? (int32_t)__fdividef(a, b) : 0;
+  int64_t left = rem - (int64_t)((uint64_t)(uint32_t)n * (uint64_t)inc);
+  n += left > 0 ? 1 : 0;
+  left -= inc;
+  while (in_time && left > 0) { ++n; left -= inc; }
+  return in_time ? n : 0;
 }
 
 // The frontier's two binary64 tests are kept out of line: inlined, the
@@ -592,13 +596,18 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     enx = A.ent_next + slot * (size_t)((cap + 3) & ~3);
   }
   int64_t *eP = A.ent_P + slot * (size_t)cap * 8;
-  __shared__ __align__(16) int64_t s_rows[WPC][32 * 8];   // the new cells' table rows
+  __shared__ __align__(16) int64_t s_rows[WPC][32 * 8];   // table rows of 32 cells
+  __shared__ __align__(16) int64_t s_prg[WPC][32 * 8];    // hour boundary: their progress
+  __shared__ int32_t s_qent[WPC][64];                     // hour boundary: kept entries
+  __shared__ uint8_t s_qam[WPC][64];                      // and their open axes
   __shared__ uint32_t s_buf[WPC][32];                     // a window's entries, crossings, burn-outs
   __shared__ uint8_t s_off[WPC][32];                      // the new cells' offsets
   __shared__ uint32_t s_dbits[WPC][LAZY ? kWinRows * kWinWords / 32 : 1];   // chunks known done this hour
   __shared__ int32_t s_claim[WPC][LAZY ? 32 : 1];
   __shared__ long long s_prof[WPC][PROF ? kProfCounters : 1];
-  int64_t *rowbuf = s_rows[wib];
+  int64_t *rowbuf = s_rows[wib], *prgbuf = s_prg[wib];
+  int32_t *qent = s_qent[wib];
+  uint8_t *qam = s_qam[wib];
   uint32_t *buf = s_buf[wib];
   uint8_t *obuf = s_off[wib];
   uint32_t *dbits = s_dbits[wib];
@@ -673,13 +682,23 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       pl.r0 = min(max(ir - kWinRows / 2, 0), max(rows - kWinRows, 0));
       pl.w0 = min(max((icc >> 5) - kWinWords / 2, 0), max(wpr - kWinWords, 0));
       need_global = rows > kWinRows || wpr > kWinWords;
+#pragma unroll 8
       for (int32_t i = lane; i < kWinRows * kWinWords; i += 32) {
         const int32_t rr = pl.r0 + i / kWinWords, ww = pl.w0 + i % kWinWords;
         pl.sav[i] = (rr < rows && ww < wpr) ? __ldg(&burnable[rr * wpr + ww]) : 0u;
       }
     }
-    if (need_global)
-      for (int32_t i = lane; i < pw; i += 32) pl.gav[i] = __ldg(&burnable[i]);
+    if (need_global) {   // eight loads in flight
+      int32_t i = lane;
+      for (; i + 7 * 32 < pw; i += 8 * 32) {
+        uint32_t v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = __ldg(&burnable[i + 32 * j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) pl.gav[i + 32 * j] = v[j];
+      }
+      for (; i < pw; i += 32) pl.gav[i] = __ldg(&burnable[i]);
+    }
     if (use_delta)
       for (int32_t i = lane; i < pw; i += 32) pl.gbr[i] = 0u;
     __syncwarp();
@@ -844,88 +863,127 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       uint64_t cal = 0;   // offsets of this hour at which some entry crosses
 
       if (prof && lane == 0) pc_t = clock64();
-      // ---- hour boundary, one lane per listed cell, 32 cells at a time:
-      // (i) drop burned-out cells and cells with no open axis (order kept);
-      // (ii) the cell's perturbation for this hour; (iii) on every open axis,
-      // the crossing period of this hour, or the progress carried to the next;
-      // (iv) the offset of its first crossing.
+      // ---- hour boundary.  (B1) drop burned-out cells and cells with no way
+      // left (order kept): one lane per listed cell, the kept ones queued up to
+      // 32; (B2) lane i takes the i-th of them: table row and progress into
+      // shared memory (asynchronously), the perturbation for this hour; (B3)
+      // one open axis per lane: the crossing period of this hour, or the
+      // progress carried to the next; (B4) the entry at its new place.
       {
-        int32_t out = 0;
-        for (int32_t b0 = 0; b0 < cnt; b0 += 32) {
-          const int32_t e = b0 + lane;
-          bool keep = false;
-          uint32_t rc = 0u, am = 0u;   // am: open axes toward Available cells
-          if (e < cnt) {
-            rc = erc[e];
-            const uint32_t m = open_axes(*reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8));
-            const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
-            uint32_t b[3];
-            pl.template block<1>(cr, cc, b);
-            am = m & axes_of_rows(b[0], b[1], b[2]);
-            // with A5 (i) a cell with no way left may still die before its neighbours are gone
-            keep = use_delta ? m != 0u && (b[0] | b[1] | b[2]) != 0u && !pl.burned(cr, cc) : am != 0u;
+        int32_t out = 0, queued = 0, b0 = 0;
+        while (b0 < cnt || queued > 0) {
+          if (b0 < cnt && queued < 32) {
+            const int32_t e = b0 + lane;
+            bool keep = false;
+            uint32_t am = 0u;   // open axes toward Available cells
+            if (e < cnt) {
+              const uint32_t rc = erc[e];
+              const uint32_t m = open_axes(*reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8));
+              const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
+              uint32_t b[3];
+              pl.template block<1>(cr, cc, b);
+              am = m & axes_of_rows(b[0], b[1], b[2]);
+              // with A5 (i) a cell with no way left may still die before its neighbours are gone
+              keep = use_delta ? m != 0u && (b[0] | b[1] | b[2]) != 0u && !pl.burned(cr, cc) : am != 0u;
+            }
+            const uint32_t bal = __ballot_sync(FULL, keep);
+            if (keep) {
+              const int32_t at = queued + __popc(bal & lt);
+              qent[at] = e;
+              qam[at] = (uint8_t)am;
+            }
+            queued += __popc(bal);
+            b0 += 32;
+            __syncwarp();
+            continue;
+          }
+          const int32_t m = min(queued, 32);
+          const bool act = lane < m;
+          uint32_t rc = 0u, am = 0u;
+          float f = 1.0f;
+          bool dies = false;
+          if (act) {
+            rc = erc[qent[lane]];
+            am = qam[lane];
           }
           const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
-          if (lazy) ensure(h, keep, cr, cc);   // this hour's row of the cell
           const int64_t cell = (int64_t)cr * cols + cc;
-          int64_t P[8], bk[8];
-          if (keep) {   // progress and rate row: 64 bytes each, four 16-byte loads
-            const longlong2 *pp = reinterpret_cast<const longlong2 *>(eP + (size_t)e * 8);
-            const longlong2 *rw = reinterpret_cast<const longlong2 *>(baseh + cell * 8);
+          if (lazy) ensure(h, act, cr, cc);   // this hour's row of the cell
+          if (act) {
+            const int64_t *row = baseh + cell * 8, *pp = eP + (size_t)qent[lane] * 8;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const longlong2 a = pp[j], b = __ldcg(rw + j);
-              P[2 * j] = a.x; P[2 * j + 1] = a.y;
-              bk[2 * j] = b.x; bk[2 * j + 1] = b.y;
+              copy_async16(rowbuf + lane * 8 + 2 * j, row + 2 * j);
+              copy_async16(prgbuf + lane * 8 + 2 * j, pp + 2 * j);
             }
             // the cell's row of the next hour into L2, for the next boundary
-            if (!LAZY && h + 1 < H) prefetch_l2(baseh + n * 8 + cell * 8);
-          } else {
-            am = 0u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) P[q] = bk[q] = 0;
+            if (!LAZY && h + 1 < H) prefetch_l2(row + n * 8);
+            f = noise_factor(seed, (uint32_t)r, (uint32_t)cell, (uint32_t)h, sigma);
+            // A5 (i): a cell whose HROS * f is below delta still sends in the
+            // first period of the hour and is Burned after it
+            if (use_delta) dies = below_delta(hrosh, cell, f, delta);
           }
-          const float f = keep ? noise_factor(seed, (uint32_t)r, (uint32_t)cell, (uint32_t)h, sigma) : 1.0f;
-          const uint64_t F = noise_fixed(f);
-          // A5 (i): a cell whose HROS * f is below delta still sends in the
-          // first period of the hour and is Burned after it
-          const bool dies = keep && use_delta && below_delta(hrosh, cell, f, delta);
-          uint64_t c8 = ~0ull;   // crossing-offset bytes
+          copy_async_wait();
+          __syncwarp();
+          // every entry of the batch has been read: its new places (never past
+          // its old ones) can be written
+          if (act) *reinterpret_cast<uint64_t *>(ecofs + (size_t)(out + lane) * 8) = ~0ull;
+          const uint32_t na = (uint32_t)__popc(am);
+          int32_t at = 0, total = 0;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            uint32_t cof = kNone;
-            if ((am >> q) & 1u) {
-              const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
-              const int64_t inc = apply_noise(bk[q], F, dq);
-              const int64_t rem = dq - P[q];
-              if (inc > 0 && inc * sph >= rem) {
-                cof = (uint32_t)(ceil_div_small(rem, inc, len_shift) - 1);
-              } else {
-                P[q] += inc * sph;
-                cof = kOpen;
-              }
-              if (dies && cof != 0u) cof = kNone;
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t bal = __ballot_sync(FULL, (na >> j) & 1u);
+            at += __popc(bal & lt) << j;
+            total += __popc(bal) << j;
+          }
+          for (int32_t t0 = 0; t0 < total; t0 += 32) {
+            while (am != 0u && at < t0 + 32) {
+              const uint32_t q = (uint32_t)(__ffs(am) - 1);
+              am &= am - 1u;
+              buf[at - t0] = (uint32_t)lane | (q << 5);
+              ++at;
             }
-            c8 = (c8 & ~(0xFFull << (8 * q))) | ((uint64_t)cof << (8 * q));
+            __syncwarp();
+            const bool valid = t0 + lane < total;
+            const uint32_t c = valid ? buf[lane] : 0u;
+            const int i = (int)(c & 31u), q = (int)(c >> 5);
+            const float fi = __shfl_sync(FULL, f, i);
+            const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
+            const int64_t inc = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
+            const int64_t P = prgbuf[i * 8 + q];
+            const int32_t np = periods_to_cross(dq - P, inc, sph, len_shift);
+            if (valid) {
+              ecofs[(size_t)(out + i) * 8 + q] = (uint8_t)(np ? (uint32_t)np - 1u : kOpen);
+              if (!np) eP[(size_t)(out + i) * 8 + q] = P + inc * sph;
+            }
+            __syncwarp();
           }
-          const bool burns = dies && pl.burn(cr, cc);
-          const uint32_t bal = __ballot_sync(FULL, keep);
-          const int32_t pos = out + __popc(bal & lt);
-          __syncwarp();   // every lane has read its entry before any slot is rewritten
           uint64_t bit = 0;
-          if (keep) {
+          bool burns = false;
+          if (act) {
+            uint64_t c8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)(out + lane) * 8);
+            if (dies) {
+              for (int q = 0; q < 8; ++q)
+                if ((c8 >> (8 * q)) & 0xFFull) c8 |= 0xFFull << (8 * q);
+              *reinterpret_cast<uint64_t *>(ecofs + (size_t)(out + lane) * 8) = c8;
+              burns = pl.burn(cr, cc);
+            }
             const uint32_t nx = min_byte8(c8);
-            erc[pos] = rc;
-            *reinterpret_cast<uint64_t *>(ecofs + (size_t)pos * 8) = c8;
-            enx[pos] = (uint8_t)nx;
-            longlong2 *pp = reinterpret_cast<longlong2 *>(eP + (size_t)pos * 8);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) pp[j] = make_longlong2(P[2 * j], P[2 * j + 1]);
+            erc[out + lane] = rc;
+            enx[out + lane] = (uint8_t)nx;
             bit = cal_bit(nx);
           }
           cal |= cal_or(bit);
-          out += __popc(bal);
           if (use_delta) dying += __popc(__ballot_sync(FULL, burns));
+          out += m;
+          queued -= m;
+          const int32_t qe = lane < queued ? qent[32 + lane] : 0;   // at most 31 are left
+          const uint8_t qa = lane < queued ? qam[32 + lane] : 0;
+          __syncwarp();
+          if (lane < queued) {
+            qent[lane] = qe;
+            qam[lane] = qa;
+          }
           __syncwarp();
         }
         cnt = out;
@@ -1069,6 +1127,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         float f = 1.0f;
         uint32_t nam = 0u;   // its axes towards Available cells | offset << 8
+        uint32_t fuel9 = 0u; // the burnable cells of the 3 x 3 block around it
         bool dies = false;
         if (act) {
           const int64_t *row = baseh + ncell * 8;
@@ -1077,6 +1136,17 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           uint32_t b[3];
           pl.template block<1>(nr, ncol, b);
           nam = axes_of_rows(b[0], b[1], b[2]) | (no << 8);
+          const int32_t wl = (ncol - 1) >> 5, wh = (ncol + 1) >> 5;
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const int32_t rr = nr - 1 + d;
+            uint32_t lo = 0u, hi = 0u;
+            if (rr >= 0 && rr < rows) {
+              if (wl >= 0) lo = __ldg(&burnable[rr * wpr + wl]);
+              if (wh < wpr) hi = __ldg(&burnable[rr * wpr + wh]);
+            }
+            fuel9 |= (__funnelshift_r(lo, hi, (uint32_t)(ncol - 1) & 31u) & 7u) << (3 * d);
+          }
           f = noise_factor(seed, (uint32_t)r, (uint32_t)ncell, (uint32_t)h, sigma);
           if (use_delta && below_delta(hrosh, ncell, f, delta)) { dies = true; nam &= ~0xFFu; }   // A5 (i)
         }
@@ -1084,22 +1154,18 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         __syncwarp();
         // (C2) four cells at a time, lane k of each 8-lane group owning axis k:
         // first crossings, progress to the end of the hour
+#pragma unroll 2
         for (int32_t b0 = 0; b0 < nc; b0 += 4) {
           const int32_t i = b0 + grp;
           const uint32_t oa = __shfl_sync(FULL, nam, i & 31);
           const float fi = __shfl_sync(FULL, f, i & 31);
-          uint32_t cof = kNone;
-          int64_t P = 0;
-          if ((oa >> k) & 1u) {
-            const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // periods left in the hour
-            const int64_t inc = apply_noise(rowbuf[i * 8 + k], noise_fixed(fi), dk);
-            cof = kOpen;
-            if (inc > 0 && inc * nmax >= dk) cof = (uint32_t)(o + ceil_div_small(dk, inc, len_shift));
-            else P = inc * nmax;
-          }
+          const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // nmax: periods left in the hour
+          const int64_t inc = apply_noise(rowbuf[(i & 31) * 8 + k], noise_fixed(fi), dk);
+          const int32_t np = periods_to_cross(dk, inc, nmax, len_shift);
+          const uint32_t cof = ((oa >> k) & 1u) ? (np ? (uint32_t)(o + np) : kOpen) : (uint32_t)kNone;
           if (i < nc) {
             ecofs[(size_t)(cnt + i) * 8 + k] = (uint8_t)cof;
-            eP[(size_t)(cnt + i) * 8 + k] = P;
+            eP[(size_t)(cnt + i) * 8 + k] = inc * nmax;   // read only while the axis is open
           }
         }
         __syncwarp();
@@ -1113,7 +1179,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         uint32_t out = 0;       // cells this lane turned Burned: count << 16 | sum of their offsets
         if (commit) pl.take(nr, ncol);
         __syncwarp();
-        uint32_t gone = 0u;     // 3 x 3 positions around the cell whose blocks hold no Available cell
+        uint32_t gone = 0u;     // burnable cells of the block around it with no Available cell around them
         if (commit) {
           uint32_t b[5];
           pl.template block<2>(nr, ncol, b);
@@ -1128,27 +1194,12 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           if (dies && pl.burn(nr, ncol)) out = (1u << 16) + no;
           const uint32_t v0 = b[0] | b[1] | b[2], v1 = b[1] | b[2] | b[3], v2 = b[2] | b[3] | b[4];
           gone = ~((v0 | (v0 >> 1) | (v0 >> 2)) & 7u | (((v1 | (v1 >> 1) | (v1 >> 2)) & 7u) << 3) |
-                   (((v2 | (v2 >> 1) | (v2 >> 2)) & 7u) << 6)) & 0x1FFu;
+                   (((v2 | (v2 >> 1) | (v2 >> 2)) & 7u) << 6)) & fuel9;
         }
         // A5 (ii): the ignited cells among them have burned out in this window
         // (a cell next to an ignition of the window had an Available neighbour
         // before it), at the last ignition next to them
         if (__any_sync(FULL, gone != 0u)) {
-          uint32_t fuel9 = 0u;   // burnable cells of the 3 x 3 positions
-          if (gone) {
-            const int32_t wl = (ncol - 1) >> 5, wh = (ncol + 1) >> 5;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-              const int32_t rr = nr - 1 + d;
-              uint32_t lo = 0u, hi = 0u;
-              if (rr >= 0 && rr < rows) {
-                if (wl >= 0) lo = __ldg(&burnable[rr * wpr + wl]);
-                if (wh < wpr) hi = __ldg(&burnable[rr * wpr + wh]);
-              }
-              fuel9 |= (__funnelshift_r(lo, hi, (uint32_t)(ncol - 1) & 31u) & 7u) << (3 * d);
-            }
-          }
-          gone &= fuel9;
           // the last cells' first: places counted from the highest lane
           const uint32_t ng = (uint32_t)__popc(gone);
           int32_t at = 0, total = 0;
@@ -1243,13 +1294,19 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     W += (long long)live * (long long)H * sph;
     {   // scar plane: burnable cells that are no longer Available
       uint32_t *dst = J.ign_plane + (size_t)r * pw;
-      for (int32_t i = lane; i < pw; i += 32) {
+      auto scar = [&](int32_t i) -> uint32_t {
         const int32_t rr = i / wpr, ww = i - rr * wpr;
-        uint32_t a;
-        if (pl.in_win(rr, ww)) a = pl.sav[(rr - pl.r0) * kWinWords + (ww - pl.w0)];
-        else a = pl.gav[i];
-        dst[i] = __ldg(&burnable[i]) & ~a;
+        return __ldg(&burnable[i]) & ~(pl.in_win(rr, ww) ? pl.sav[(rr - pl.r0) * kWinWords + (ww - pl.w0)] : pl.gav[i]);
+      };
+      int32_t i = lane;
+      for (; i + 3 * 32 < pw; i += 4 * 32) {   // four words in flight
+        uint32_t v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = scar(i + 32 * j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dst[i + 32 * j] = v[j];
       }
+      for (; i < pw; i += 32) dst[i] = scar(i);
     }
     if (lane == 0) {
       if (A.trace.rec) trace_record(A.trace, kTraceReplica, (uint32_t)r, J.trace_tag, t_start, global_ns());
