@@ -167,20 +167,37 @@ __device__ inline void cell_prep(double gs, double aspect_deg, CellPrep *cp) {
   dsincos_deg(__dadd_rn(aspect_deg, 180.0), &cp->sin_s, &cp->cos_s);
 }
 
-struct FbpOut { double hros, bros, lb, fros, a, e, ux, uy, wsv, wse; double ros[8]; };
+// HROS and the 8 axis rates of a cell and hour (m/min).  Under Eq. (1) the
+// axes come in four opposite pairs, of which one has the rate `back` common to
+// all axes that do not point ahead: `paired` rows hold the other rate of pair j
+// (axes j and j + 4) in ros[j], and bit j of `behind` says that it is axis
+// j + 4's; other rows hold all 8 in ros.
+struct AxisRates {
+  double hros, back;
+  uint32_t behind;
+  bool paired;
+  double ros[8];
+  __device__ __forceinline__ double of(int k) const {
+    if (!paired) return ros[k];
+    return (((behind >> (k & 3)) & 1u) != 0u) == (k >= 4) ? ros[k & 3] : back;
+  }
+};
+
+// half of a non-negative number, by its exponent while it stays normal
+__device__ __forceinline__ double halved(double x) {
+  const uint64_t b = bits_of(x);
+  return (uint32_t)(b >> 32) - 0x00200000u < 0x7FD00000u ? double_of(b - 0x0010000000000000ull) : __dmul_rn(x, 0.5);
+}
 
 // Sec. 3.7, Eqs. (2)-(4): the ellipse of a cell from HROS, BROS and LB, and
 // its rate along each of the 8 axes for the head direction (ux, uy) (unit
 // vector, x east, y north) by Eq. (1) (ellipse_mode 0) or by the ray from the
-// ignition point (mode 1).  Sets o->lb, fros, a, e, ux, uy and ros[].
+// ignition point (mode 1).
 __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb, double ux, double uy,
-                                             int ellipse_mode, FbpOut *o) {
+                                             int ellipse_mode, AxisRates *o) {
   const double hb = __dadd_rn(hros, bros);
-  const double ilb = __ddiv_rn(1.0, lb);   // one reciprocal for FROS and e
-  const double fros = __dmul_rn(__dmul_rn(hb, ilb), 0.5);
-  const double a = __dmul_rn(hb, 0.5);
-  const double e = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(ilb, ilb)));
-  o->lb = lb; o->fros = fros; o->a = a; o->e = e; o->ux = ux; o->uy = uy;
+  const double ilb = ddiv(1.0, lb);   // one reciprocal for FROS and e
+  const double a = halved(hb);
   // cos(phi_k) = (cos theta_k) ux + (sin theta_k) uy for the 8 axes, whose
   // cosines and sines are 0, +-1 and +-h (h = RN(sqrt(1/2))): products by 0 and
   // +-1 are exact, so the sums are ux, uy, their negatives and +-(h ux) +- (h uy)
@@ -188,14 +205,20 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
   const double h = 0x1.6a09e667f3bcdp-1;
   const double hx = __dmul_rn(h, ux), hy = __dmul_rn(h, uy);
   const double dpp = __dadd_rn(hx, hy), dmp = __dsub_rn(hy, hx);
-  const double cphk[8] = {ux, dpp, uy, dmp, -ux, -dpp, -uy, -dmp};
+  o->hros = hros;
   if (ellipse_mode == 0) {
+    const double e = droot(__dsub_rn(1.0, __dmul_rn(ilb, ilb)));
     const double A = __dmul_rn(a, __dsub_rn(1.0, __dmul_rn(e, e)));
+    const double cph[4] = {ux, dpp, uy, dmp};
+    o->back = A;
+    o->paired = true;
+    o->behind = 0u;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const double cphi = cphk[k];
-      // cphi > 0 as a sign test on the bits (cphi is never NaN)
-      o->ros[k] = (__double_as_longlong(cphi) > 0) ? __ddiv_rn(A, __dsub_rn(1.0, __dmul_rn(e, cphi))) : A;
+    for (int j = 0; j < 4; ++j) {   // one of the axes j and j + 4 points ahead (neither at cos = 0)
+      const uint64_t c = bits_of(cph[j]);
+      const double ahead = double_of(c & 0x7FFFFFFFFFFFFFFFull);
+      o->behind |= (uint32_t)(c >> 63) << j;
+      o->ros[j] = pos(ahead) ? ddiv(A, __dsub_rn(1.0, __dmul_rn(e, ahead))) : A;
     }
   } else {
     // the ray from the ignition point, c = (HROS - BROS)/2 behind the centre,
@@ -205,10 +228,12 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
     // on the back half (cos < 0), the same ray multiplied out by the conjugate
     // of its numerator, r = b^2 HROS BROS / (a b sqrt(Q) - b^2 c cos), so that
     // no nearly equal terms are subtracted when HROS >> BROS
-    const double b = fros;
+    const double b = halved(__dmul_rn(hb, ilb));   // FROS
     const double c = __dmul_rn(__dsub_rn(hros, bros), 0.5);
     const double hbp = __dmul_rn(hros, bros);
     const double bb = __dmul_rn(b, b), aa = __dmul_rn(a, a), ab = __dmul_rn(a, b);
+    const double cphk[8] = {ux, dpp, uy, dmp, -ux, -dpp, -uy, -dmp};
+    o->paired = false;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const double cphi = cphk[k];
@@ -216,13 +241,13 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
       if (sphi2 < 0.0) sphi2 = 0.0;
       const double bc = __dmul_rn(__dmul_rn(bb, cphi), cphi);
       const double den = __dadd_rn(bc, __dmul_rn(aa, sphi2));
-      const double root = __dsqrt_rn(__dadd_rn(bc, __dmul_rn(hbp, sphi2)));
+      const double root = droot(__dadd_rn(bc, __dmul_rn(hbp, sphi2)));
       double r = 0.0;
       if (cphi >= 0.0) {
-        if (den > 0.0) r = __ddiv_rn(__dadd_rn(__dmul_rn(__dmul_rn(bb, c), cphi), __dmul_rn(ab, root)), den);
+        if (den > 0.0) r = ddiv(__dadd_rn(__dmul_rn(__dmul_rn(bb, c), cphi), __dmul_rn(ab, root)), den);
       } else {
         const double q = __dsub_rn(__dmul_rn(ab, root), __dmul_rn(__dmul_rn(bb, c), cphi));
-        if (q > 0.0) r = __ddiv_rn(__dmul_rn(bb, hbp), q);
+        if (q > 0.0) r = ddiv(__dmul_rn(bb, hbp), q);
       }
       o->ros[k] = r;
     }
@@ -232,7 +257,7 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
 // per (cell, hour): FBP surface spread, Eqs. (2)-(4), then the 8 axis rates
 // by Eq. (1) (ellipse_mode 0) or by the centre-offset ellipse ray (mode 1).
 __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const HourPrep &hp,
-                               double pcf, int ellipse_mode, FbpOut *o) {
+                               double pcf, int ellipse_mode, AxisRates *o) {
   const double cf = hp.cf;
   double wse = 0.0;
   if (pos(gs)) {
@@ -250,10 +275,10 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
   }
   const double wsx = __dadd_rn(hp.wsx_w, __dmul_rn(wse, cp.sin_s));
   const double wsy = __dadd_rn(hp.wsy_w, __dmul_rn(wse, cp.cos_s));
-  const double wsv = __dsqrt_rn(__dadd_rn(__dmul_rn(wsx, wsx), __dmul_rn(wsy, wsy)));
+  const double wsv = droot(__dadd_rn(__dmul_rn(wsx, wsx), __dmul_rn(wsy, wsy)));
   double ux = 1.0, uy = 0.0;
   if (pos(wsv)) {
-    const double iw = __ddiv_rn(1.0, wsv);
+    const double iw = ddiv(1.0, wsv);
     ux = __dmul_rn(wsx, iw);
     uy = __dmul_rn(wsy, iw);
   }
@@ -267,16 +292,37 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
     lb = !lt_c(wsv, 1.0) ? __dmul_rn(1.1, dpow_n2(wsv, 0.464, 0)) : 1.0;
   else
     lb = __dadd_rn(1.0, __dmul_rn(8.729, dpow_n2(__dsub_rn(1.0, dexp(__dmul_rn(-0.030, wsv))), 2.155, 0)));
-  o->hros = hros; o->bros = bros; o->wsv = wsv; o->wse = wse;
   ellipse_axes(hros, bros, lb, ux, uy, ellipse_mode, o);
 }
 
-// 2^32 fixed point of a non-negative real: 0 for non-positive / NaN, capped at
-// 2^62.  The conversion saturates (and gives INT64_MIN for NaN), so clamping
-// the integer gives the same result as testing x first, without FP64 compares.
-__device__ __forceinline__ int64_t fixed_of(double x) {
-  const long long v = __double2ll_rn(x);
-  return v <= 0 ? 0 : (v >= 4611686018427387904LL ? 4611686018427387904LL : (int64_t)v);
+// the integer nearest to x 2^up (ties to even) for a non-negative real, by
+// shifts: 0 for non-positive / NaN, capped at 2^62
+__device__ __forceinline__ int64_t fixed_of(double x, int up) {
+  const uint64_t b = bits_of(x);
+  if (b > 0x7FF0000000000000ull) return 0;
+  const int s = (int)(b >> 52) - 1075 + up;
+  const uint64_t m = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  if (s >= 10) return 4611686018427387904ll;   // m >= 2^52
+  if (s >= 0) return (int64_t)(m << s);
+  if (s < -53) return 0;                       // below 1/2
+  const uint64_t q = m >> -s, rest = m << (64 + s);
+  return (int64_t)(q + ((rest > 0x8000000000000000ull || (rest == 0x8000000000000000ull && (q & 1))) ? 1 : 0));
 }
+
+// the factor dt 2^32 of the per-period increments: a power of two (dt = 1, 2,
+// 4) is exact and only moves the exponent, any other rounds the product first
+struct PeriodScale {
+  double factor;
+  int up;
+  __device__ __forceinline__ explicit PeriodScale(double dt2p32) {
+    const uint64_t b = bits_of(dt2p32);
+    const bool exact = (b & 0x000FFFFFFFFFFFFFull) == 0;
+    factor = exact ? 0.0 : dt2p32;
+    up = exact ? (int)(b >> 52) - 1023 : 0;
+  }
+  __device__ __forceinline__ int64_t operator()(double ros) const {
+    return up ? fixed_of(ros, up) : fixed_of(__dmul_rn(ros, factor), 0);
+  }
+};
 
 }  // namespace c2f

@@ -209,40 +209,47 @@ __global__ void k_order_scatter(const uint8_t *fuel, const float *slope, const u
 // (const_ros > 0: the deterministic test rates -- all 8 axes at const_ros, or,
 // with const_bros > 0 or const_lb > 1, the ellipse of HROS = const_ros,
 // BROS = const_bros (0: const_ros), LB = const_lb headed along the hour's wind)
-__device__ __forceinline__ double row_rates(int fuel, const float *slope, int64_t cell,
-                                            const CellPrep &cp, const HourPrep &hp, double pcf,
-                                            double const_ros, double const_bros, double const_lb,
-                                            int ellipse_mode, double ros[8]) {
+__device__ __forceinline__ void row_rates(int fuel, const float *slope, int64_t cell,
+                                          const CellPrep &cp, const HourPrep &hp, double pcf,
+                                          double const_ros, double const_bros, double const_lb,
+                                          int ellipse_mode, AxisRates *o) {
   if (pos(const_ros)) {
     if (pos(const_bros) || gt_c(const_lb, 1.0)) {
-      FbpOut o;
       ellipse_axes(const_ros, pos(const_bros) ? const_bros : const_ros, gt_c(const_lb, 1.0) ? const_lb : 1.0,
-                   hp.sin_w, hp.cos_w, ellipse_mode, &o);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) ros[k] = o.ros[k];
-      return const_ros;
+                   hp.sin_w, hp.cos_w, ellipse_mode, o);
+      return;
     }
+    o->hros = const_ros;
+    o->paired = false;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) ros[k] = const_ros;
-    return const_ros;
+    for (int k = 0; k < 8; ++k) o->ros[k] = const_ros;
+    return;
   }
-  const double gs = slope ? (double)slope[cell] : 0.0;
-  FbpOut o;
-  fbp_row(fuel, gs, cp, hp, pcf, ellipse_mode, &o);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) ros[k] = o.ros[k];
-  return o.hros;
+  fbp_row(fuel, slope ? (double)slope[cell] : 0.0, cp, hp, pcf, ellipse_mode, o);
 }
 
 // a table row: the 8 per-period increments B_k = fixed(ros_k * dt * 2^32) in one
 // 64-byte line (four 16-byte stores), HROS beside it in its own array
-__device__ __forceinline__ void row_store(int64_t *row, double *hros_at, const double ros[8],
-                                          double hr, double dt2p32) {
+__device__ __forceinline__ void row_store(int64_t *row, double *hros_at, const AxisRates &o, double dt2p32) {
+  const PeriodScale fixed(dt2p32);
+  int64_t v[8];
+  if (o.paired) {
+    const int64_t back = fixed(o.back);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int64_t ahead = fixed(o.ros[j]);
+      const bool behind = (o.behind >> j) & 1u;
+      v[j] = behind ? back : ahead;
+      v[j + 4] = behind ? ahead : back;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = fixed(o.ros[k]);
+  }
   longlong2 *dst = reinterpret_cast<longlong2 *>(row);
 #pragma unroll
-  for (int k = 0; k < 8; k += 2)
-    dst[k / 2] = make_longlong2(fixed_of(__dmul_rn(ros[k], dt2p32)), fixed_of(__dmul_rn(ros[k + 1], dt2p32)));
-  *hros_at = hr;
+  for (int k = 0; k < 8; k += 2) dst[k / 2] = make_longlong2(v[k], v[k + 1]);
+  *hros_at = o.hros;
 }
 
 // nanoseconds of the GPU's global timer
@@ -277,25 +284,21 @@ __global__ void __launch_bounds__(128) k_ros_table(RosTableArgs a) {
   const int h = a.hour0 + blockIdx.y;
   const int32_t row = (int32_t)(cell / a.cols), col = (int32_t)(cell % a.cols);
   const bool burn = (a.burnable[(int64_t)row * a.wpr + (col >> 5)] >> (col & 31)) & 1u;
-  double ros[8];
-  double hr = 0.0;
-  if (!burn) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) ros[k] = 0.0;
-  } else {
-    hr = row_rates(a.fuel[cell], a.slope, cell, a.cell[cell], a.hour[h], a.pcf, a.const_ros,
-                   a.const_bros, a.const_lb, a.ellipse_mode, ros);
-  }
   const size_t idx = (size_t)h * n + cell;
-  if (a.base) {
-    double scratch;
-    row_store(a.base + idx * 8, a.hros ? a.hros + idx : &scratch, ros, hr, a.dt2p32);
-  } else if (a.hros) {
-    a.hros[idx] = hr;
+  AxisRates o;
+  if (burn) {
+    row_rates(a.fuel[cell], a.slope, cell, a.cell[cell], a.hour[h], a.pcf, a.const_ros, a.const_bros, a.const_lb,
+              a.ellipse_mode, &o);
+    if (a.base) row_store(a.base + idx * 8, a.hros + idx, o, a.dt2p32);
+  } else if (a.base) {
+    longlong2 *dst = reinterpret_cast<longlong2 *>(a.base + idx * 8);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dst[k] = make_longlong2(0, 0);
+    a.hros[idx] = 0.0;
   }
   if (a.ros8) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a.ros8[(size_t)cell * 8 + k] = ros[k];
+    for (int k = 0; k < 8; ++k) a.ros8[(size_t)cell * 8 + k] = burn ? o.of(k) : 0.0;
   }
   if (traced) trace_record(a.trace, kTraceTable, (uint32_t)h, a.trace.tag, t_start, global_ns());
 }
@@ -419,11 +422,11 @@ __device__ __forceinline__ void table_chunk(const SimJob &J, int32_t h, int32_t 
   if (col < J.cols && ((__ldg(&J.burnable[w]) >> lane) & 1u)) {
     const int64_t n = (int64_t)J.rows * J.cols;
     const int64_t cell = (int64_t)row * J.cols + col;
-    double ros[8];
-    const double hr = row_rates(__ldg(&J.fuel[cell]), J.slope, cell, J.cell[cell], J.hour[h], J.pcf,
-                                J.const_ros, J.const_bros, J.const_lb, J.ellipse_mode, ros);
+    AxisRates o;
+    row_rates(__ldg(&J.fuel[cell]), J.slope, cell, J.cell[cell], J.hour[h], J.pcf, J.const_ros, J.const_bros,
+              J.const_lb, J.ellipse_mode, &o);
     const size_t idx = (size_t)h * n + cell;
-    row_store(J.base + idx * 8, J.hros + idx, ros, hr, J.dt2p32);
+    row_store(J.base + idx * 8, J.hros + idx, o, J.dt2p32);
   }
   __threadfence();
   __syncwarp();

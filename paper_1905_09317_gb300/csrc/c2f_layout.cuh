@@ -138,7 +138,7 @@ struct RosTableArgs {
   double pcf, const_ros, const_bros, const_lb, dt2p32;
   int32_t ellipse_mode;
   int64_t *base;           // [hour][N][8] (absolute hour), or nullptr
-  double *hros;            // [hour][N], or nullptr
+  double *hros;            // [hour][N] with base
   double *ros8;            // export: [N][8] of hour0 only, or nullptr
   const int32_t *order;    // cells grouped by (fuel code, sloped); nullptr = identity
   TraceArgs trace;         // one record per CTA when on

@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "c2f_exact.cuh"
 #include "c2f_layout.cuh"
 
 namespace c2f {
@@ -91,6 +92,21 @@ __device__ __forceinline__ double scale2(double p, int k) {
   return __dmul_rn(p, pow2i(k));
 }
 
+// x / y and sqrt(x), correctly rounded: on the integer units over the range
+// that the rates take, by the FP64 instructions elsewhere
+__device__ __noinline__ double ddiv_any(double x, double y) { return __ddiv_rn(x, y); }
+__device__ __noinline__ double dsqrt_any(double x) { return __dsqrt_rn(x); }
+__device__ __forceinline__ double ddiv(double x, double y) {
+  return mid_range(bits_of(x)) && mid_range(bits_of(y)) ? div_mid(x, y) : ddiv_any(x, y);
+}
+__device__ __forceinline__ double droot(double x) { return mid_range(bits_of(x)) ? sqrt_mid(x) : dsqrt_any(x); }
+
+// a binary32 integer as binary64, by its bits
+__device__ __forceinline__ double widen_int(float f) {
+  const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+  return __hiloint2double(a ? (int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)) : 0, (int)(u << 29));
+}
+
 __device__ inline double dexp_series(double x) {
   // |x| < 704 (integer test of the high word) skips the range checks below
   if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) {
@@ -134,20 +150,33 @@ __device__ inline double dlog_series(double x) {
 }
 
 __device__ inline double dexp(double x) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) {   // |x| >= 704
+  const uint32_t hx = (uint32_t)__double2hiint(x), ax = hx & 0x7fffffffu;
+  if (ax >= 0x40860000u) {   // |x| >= 704
     if (x != x) return x;
     if (x > 709.78) return __longlong_as_double(0x7ff0000000000000LL);
     if (x < -745.2) return 0.0;
   }
-  const double kd = rint(__dmul_rn(x, kInvLn2 * 64.0));
+  // kd = rint(RN(x 64/ln2)), found in binary32 off the FP64 pipe: x truncated
+  // to 24 bits and two roundings leave the product within 2^-21 of itself, so
+  // unless it lies that close to a half the nearest integer is the same
+  const float xf = ax < 0x38100000u
+      ? 0.0f : __uint_as_float((hx & 0x80000000u) | ((ax - 0x38000000u) << 3) | ((uint32_t)__double2loint(x) >> 29));
+  const float t32 = __fmul_rn(xf, (float)(kInvLn2 * 64.0));
+  const float s32 = __fadd_rn(t32, 12582912.0f);   // 1.5 2^23: rounds to an integer, |t32| < 2^17
+  const float kf = __fsub_rn(s32, 12582912.0f);
+  int k = __float_as_int(s32) - 0x4B400000;
+  double kd = widen_int(kf);
+  if (!(fabsf(__fsub_rn(t32, kf)) < 0.4999f - fabsf(t32) * 0x1p-21f) || ax >= 0x40860000u) {
+    kd = rint(__dmul_rn(x, kInvLn2 * 64.0));
+    k = (int)kd;
+  }
   const double r = __fma_rn(-kd, kLn2Lo / 64.0, __fma_rn(-kd, kLn2Hi / 64.0, x));
   double q = __fma_rn(__fma_rn(g_mc.inv_fact[5], r, g_mc.inv_fact[4]), r, g_mc.inv_fact[3]);
   q = __fma_rn(q, r, g_mc.inv_fact[2]);
   const double p = __fma_rn(q, __dmul_rn(r, r), r);   // exp(r) - 1 to r^5
-  const long long k = (long long)kd;
   const double t = __ldg(&g_exp_tab[k & 63]);
   const double y = __fma_rn(t, p, t);                  // in [2^(-1/128), 2)
-  const int m = (int)(k >> 6);
+  const int m = k >> 6;
   // y 2^m is exact while it stays normal: add m to the exponent field
   if (m >= -1020 && m <= 1022) return __longlong_as_double(__double_as_longlong(y) + ((long long)m << 52));
   return scale2(y, m);
@@ -176,8 +205,9 @@ __device__ inline double dlog(double x) {
   q = __fma_rn(q, r, g_mc.log_c[1]);        // 1/3
   q = __fma_rn(q, r, -0.5);
   const double lp = __fma_rn(q, __dmul_rn(r, r), r);
-  const double ed = (double)e;
-  const double hi = __dadd_rn(__dmul_rn(ed, kLn2Hi), __ldg(&g_log_tab[j]));
+  const double ed = widen_int((float)e);
+  // e kLn2Hi is exact (11 and 29 bits), so the fused sum rounds once, as the separate one
+  const double hi = __fma_rn(ed, kLn2Hi, __ldg(&g_log_tab[j]));
   const double lo = __fma_rn(ed, kLn2Lo, lp);
   return __dadd_rn(hi, lo);
 }
@@ -213,7 +243,7 @@ __device__ inline double dpow_n2(double x, double y, int n2) {
         r = x;
         for (int i = 1; i < n; ++i) r = __dmul_rn(r, x);
       }
-      if (n2 & 1) r = (n > 0) ? __dmul_rn(r, __dsqrt_rn(x)) : __dsqrt_rn(x);
+      if (n2 & 1) r = (n > 0) ? __dmul_rn(r, droot(x)) : droot(x);
       return r;
     }
     return dexp(__dmul_rn(y, dlog(x)));
