@@ -142,4 +142,60 @@ C2F_HD double sqrt_mid(double x) {
   return double_of((uint64_t)q + ((uint64_t)((e + 1021u) >> 1) << 52));
 }
 
+// ---- the Horner steps of exp and log
+// q = c + p r for a p of 53 bits and |r| < 2^-7, each sum rounded to binary64:
+// the exponents of every c and q are known ahead, so with r as a 64-bit integer
+// A 2^-70 (exact for |r| >= 2^-18) a step is the high part of one product, at
+// 17 to 19 bits below the sum's last place, rounded and added to c's
+// significand.  The dropped parts are under 3 units of the product's last
+// place, so a step is exact unless those bits lie within 3 of a half; then (one
+// argument in 20,000), and for smaller r, `exact` stays false and the caller
+// takes the FP64 instructions.
+struct HornerArg {
+  uint32_t a1, a0;
+  bool exact;
+  C2F_HD explicit HornerArg(double r) {
+    const uint64_t b = bits_of(r);
+    const uint32_t e = (uint32_t)(b >> 52) & 0x7FFu;
+    exact = e - 1005u <= 10u;
+    const uint64_t a = ((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << ((e - 1005u) & 15u);
+    a1 = (uint32_t)(a >> 32);
+    a0 = (uint32_t)a;
+  }
+  // round(n A 2^-(53 + guard)) for a 53-bit n
+  C2F_HD uint64_t times(uint64_t n, int guard) {
+    const uint32_t n1 = (uint32_t)(n >> 21), n0 = (uint32_t)(n << 11), half = 1u << (guard - 1);
+    const uint64_t x = wide(n1, a1) + mul_hi(n1, a0) + mul_hi(n0, a1) + half;
+    exact = exact && (((uint32_t)x + 3u) & (2u * half - 1u)) > 3u;
+    return x >> guard;
+  }
+};
+
+// significands of the constants, and the bits of 1/2
+constexpr uint64_t kM1_120 = 0x11111111111111ull, kM1_24 = 0x15555555555555ull;   // 2^-59, 2^-57
+constexpr uint64_t kM1_6 = 0x15555555555555ull, kM1_5 = 0x1999999999999Aull;      // 2^-55, 2^-55
+constexpr uint64_t kM1_3 = 0x15555555555555ull, kBitsHalf = 0x3FE0000000000000ull;   // 2^-54
+
+// ((1/120 r + 1/24) r + 1/6) r + 1/2
+C2F_HD double exp_steps(double r, bool *exact) {
+  HornerArg A(r);
+  const bool neg = (bits_of(r) >> 63) != 0;
+  const uint64_t x1 = A.times(kM1_120, 19), n1 = neg ? kM1_24 - x1 : kM1_24 + x1;
+  const uint64_t x2 = A.times(n1, 19), n2 = neg ? kM1_6 - x2 : kM1_6 + x2;
+  const uint64_t x3 = A.times(n2, neg ? 18 : 19);   // below 1/2 the last place is half as large
+  *exact = A.exact;
+  return double_of(neg ? kBitsHalf - x3 : kBitsHalf + x3);
+}
+
+// (((-1/6 r + 1/5) r - 1/4) r + 1/3) r - 1/2, for r > 0
+C2F_HD double log_steps(double r, bool *exact) {
+  HornerArg A(r);
+  const uint64_t n1 = kM1_5 - A.times(kM1_6, 17);
+  const uint64_t n2 = 0x20000000000000ull - A.times(n1, 17);   // 1/4 = 2^53 2^-55
+  const uint64_t n3 = kM1_3 - A.times(n2, 18);
+  const uint64_t x4 = A.times(n3, 17);
+  *exact = A.exact && (bits_of(r) >> 63) == 0;
+  return double_of(0x8000000000000000ull | (kBitsHalf - x4));
+}
+
 }  // namespace c2f

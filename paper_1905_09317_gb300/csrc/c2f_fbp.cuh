@@ -103,10 +103,16 @@ __device__ inline double isf_of(int fuel, const HourPrep &hp, double sf, double 
   return isf_curve(g_fuel[fuel], hp.inv_a[fuel], rsf);
 }
 
-// wind function of the ISI; above 40 km/h the saturating branch of the 2009 update
-__device__ __forceinline__ double wind_fn(double w) {
-  if (le_c(w, 40.0)) return dexp(__dmul_rn(0.05039, w));
-  return __dmul_rn(12.0, __dsub_rn(1.0, dexp(__dmul_rn(-0.0818, __dsub_rn(w, 28.0)))));
+// wind function of the ISI, up to 40 km/h and in the saturating branch of the 2009 update above,
+// and the back rate's exp(-0.05039 w)
+__device__ __forceinline__ void wind_fn(double w, double *ahead, double *back) {
+  const double x = __dmul_rn(0.05039, w);
+  if (le_c(w, 40.0)) {
+    dexp_both(x, ahead, back);
+    return;
+  }
+  *ahead = __dmul_rn(12.0, __dsub_rn(1.0, dexp(__dmul_rn(-0.0818, __dsub_rn(w, 28.0)))));
+  *back = dexp(-x);
 }
 
 // per weather hour: (ws, wd_from, ffmc, bui) -> HourPrep
@@ -186,7 +192,7 @@ struct AxisRates {
 // half of a non-negative number, by its exponent while it stays normal
 __device__ __forceinline__ double halved(double x) {
   const uint64_t b = bits_of(x);
-  return (uint32_t)(b >> 32) - 0x00200000u < 0x7FD00000u ? double_of(b - 0x0010000000000000ull) : __dmul_rn(x, 0.5);
+  return (uint32_t)(b >> 32) - 0x00200000u < 0x7FD00000u ? double_of(b - 0x0010000000000000ull) : dmul_any(x, 0.5);
 }
 
 // Sec. 3.7, Eqs. (2)-(4): the ellipse of a cell from HROS, BROS and LB, and
@@ -282,10 +288,12 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
     ux = __dmul_rn(wsx, iw);
     uy = __dmul_rn(wsy, iw);
   }
-  const double isi = __dmul_rn(hp.isz, wind_fn(wsv));
+  double fw, fb;
+  wind_fn(wsv, &fw, &fb);
+  const double isi = __dmul_rn(hp.isz, fw);
   const double be = hp.be[fuel];
   const double hros = __dmul_rn(rsi_of(fuel, isi, pcf, cf), be);
-  const double bisi = __dmul_rn(hp.isz, dexp(__dmul_rn(-0.05039, wsv)));
+  const double bisi = __dmul_rn(hp.isz, fb);
   const double bros = __dmul_rn(rsi_of(fuel, bisi, pcf, cf), be);
   double lb;
   if (is_o1(fuel))
@@ -321,7 +329,7 @@ struct PeriodScale {
     up = exact ? (int)(b >> 52) - 1023 : 0;
   }
   __device__ __forceinline__ int64_t operator()(double ros) const {
-    return up ? fixed_of(ros, up) : fixed_of(__dmul_rn(ros, factor), 0);
+    return fixed_of(up ? ros : dmul_any(ros, factor), up);
   }
 };
 

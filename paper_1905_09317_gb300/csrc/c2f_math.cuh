@@ -92,10 +92,33 @@ __device__ __forceinline__ double scale2(double p, int k) {
   return __dmul_rn(p, pow2i(k));
 }
 
-// x / y and sqrt(x), correctly rounded: on the integer units over the range
-// that the rates take, by the FP64 instructions elsewhere
+// The rare FP64 steps of the routines below, out of line: inlined, the compiler
+// predicates them instead of branching, and a predicated-off FP64 instruction
+// takes its slot of the pipe all the same (the table kernel went from 180 only
+// to 175 FP64 instructions a cell-hour when its exp and log steps moved to
+// integers with the FP64 steps kept inline behind a test).
 __device__ __noinline__ double ddiv_any(double x, double y) { return __ddiv_rn(x, y); }
 __device__ __noinline__ double dsqrt_any(double x) { return __dsqrt_rn(x); }
+__device__ __noinline__ double dmul_any(double x, double y) { return __dmul_rn(x, y); }
+__device__ __noinline__ double dscale_any(double p, int k) { return scale2(p, k); }
+__device__ __noinline__ double drint_product(double x, double y) { return rint(__dmul_rn(x, y)); }
+__device__ __noinline__ double exp_steps_any(double r) {
+  return __fma_rn(__fma_rn(__fma_rn(g_mc.inv_fact[5], r, g_mc.inv_fact[4]), r, g_mc.inv_fact[3]), r, g_mc.inv_fact[2]);
+}
+__device__ __noinline__ double log_steps_any(double r) {
+  double q = __fma_rn(-g_mc.inv_fact[3], r, g_mc.log_c[2]);   // -1/6, 1/5
+  q = __fma_rn(q, r, -0.25);
+  q = __fma_rn(q, r, g_mc.log_c[1]);                          // 1/3
+  return __fma_rn(q, r, -0.5);
+}
+__device__ __noinline__ double dexp_far(double x) {   // |x| >= 704 and not in (704, 709.78]: the value, else 1
+  if (x != x) return x;
+  if (x > 709.78) return __longlong_as_double(0x7ff0000000000000LL);
+  return x < -745.2 ? 0.0 : 1.0;
+}
+
+// x / y and sqrt(x), correctly rounded: on the integer units over the range
+// that the rates take, by the FP64 instructions elsewhere
 __device__ __forceinline__ double ddiv(double x, double y) {
   return mid_range(bits_of(x)) && mid_range(bits_of(y)) ? div_mid(x, y) : ddiv_any(x, y);
 }
@@ -149,67 +172,92 @@ __device__ inline double dlog_series(double x) {
   return __dadd_rn(__dmul_rn(ed, kLn2Hi), __fma_rn(ed, kLn2Lo, lm));
 }
 
-__device__ inline double dexp(double x) {
+// exp's argument reduction, |x| < 704: k = rint(RN(x 64/ln2)) and r = x - k
+// ln2/64 by two fused steps.  k is found in binary32 off the FP64 pipe: x
+// truncated to 24 bits and two roundings leave the product within 2^-21 of
+// itself, so unless it lies that close to a half the nearest integer is the same.
+__device__ __forceinline__ double exp_reduce(double x, int *k_out) {
   const uint32_t hx = (uint32_t)__double2hiint(x), ax = hx & 0x7fffffffu;
-  if (ax >= 0x40860000u) {   // |x| >= 704
-    if (x != x) return x;
-    if (x > 709.78) return __longlong_as_double(0x7ff0000000000000LL);
-    if (x < -745.2) return 0.0;
-  }
-  // kd = rint(RN(x 64/ln2)), found in binary32 off the FP64 pipe: x truncated
-  // to 24 bits and two roundings leave the product within 2^-21 of itself, so
-  // unless it lies that close to a half the nearest integer is the same
   const float xf = ax < 0x38100000u
       ? 0.0f : __uint_as_float((hx & 0x80000000u) | ((ax - 0x38000000u) << 3) | ((uint32_t)__double2loint(x) >> 29));
-  const float t32 = __fmul_rn(xf, (float)(kInvLn2 * 64.0));
-  const float s32 = __fadd_rn(t32, 12582912.0f);   // 1.5 2^23: rounds to an integer, |t32| < 2^17
-  const float kf = __fsub_rn(s32, 12582912.0f);
-  int k = __float_as_int(s32) - 0x4B400000;
+  const float t = __fmul_rn(xf, (float)(kInvLn2 * 64.0));
+  const float s = __fadd_rn(t, 12582912.0f);   // 1.5 2^23: rounds to an integer, |t| < 2^17
+  const float kf = __fsub_rn(s, 12582912.0f);
+  int k = __float_as_int(s) - 0x4B400000;
   double kd = widen_int(kf);
-  if (!(fabsf(__fsub_rn(t32, kf)) < 0.4999f - fabsf(t32) * 0x1p-21f) || ax >= 0x40860000u) {
-    kd = rint(__dmul_rn(x, kInvLn2 * 64.0));
+  if (!(fabsf(__fsub_rn(t, kf)) < 0.4999f - fabsf(t) * 0x1p-21f)) {
+    kd = drint_product(x, kInvLn2 * 64.0);
     k = (int)kd;
   }
-  const double r = __fma_rn(-kd, kLn2Lo / 64.0, __fma_rn(-kd, kLn2Hi / 64.0, x));
-  double q = __fma_rn(__fma_rn(g_mc.inv_fact[5], r, g_mc.inv_fact[4]), r, g_mc.inv_fact[3]);
-  q = __fma_rn(q, r, g_mc.inv_fact[2]);
-  const double p = __fma_rn(q, __dmul_rn(r, r), r);   // exp(r) - 1 to r^5
+  *k_out = k;
+  return __fma_rn(-kd, kLn2Lo / 64.0, __fma_rn(-kd, kLn2Hi / 64.0, x));
+}
+
+// 2^(k/64) exp(r), r2 = RN(r r)
+__device__ __forceinline__ double exp_finish(double r, double r2, int k) {
+  bool exact;
+  double q = exp_steps(r, &exact);
+  if (!exact) q = exp_steps_any(r);
+  const double p = __fma_rn(q, r2, r);   // exp(r) - 1 to r^5
   const double t = __ldg(&g_exp_tab[k & 63]);
   const double y = __fma_rn(t, p, t);                  // in [2^(-1/128), 2)
   const int m = k >> 6;
   // y 2^m is exact while it stays normal: add m to the exponent field
   if (m >= -1020 && m <= 1022) return __longlong_as_double(__double_as_longlong(y) + ((long long)m << 52));
-  return scale2(y, m);
+  return dscale_any(y, m);
 }
 
-__device__ inline double dlog(double x) {
-  int e = 0;
-  const int hx = __double2hiint(x);
-  if (hx < 0x00100000 || hx >= 0x7ff00000) {   // not a positive normal finite number
-    if (x != x) return x;
-    if (x < 0.0) return __longlong_as_double(0x7ff8000000000000LL);
-    if (x == 0.0) return __longlong_as_double((long long)0xfff0000000000000ULL);
-    if (__double_as_longlong(x) == 0x7ff0000000000000LL) return x;
-    if (x < 0x1p-1022) { x = __dmul_rn(x, 0x1p54); e = -54; }
+__device__ inline double dexp(double x) {
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) {   // |x| >= 704
+    const double far = dexp_far(x);
+    if (bits_of(far) != bits_of(1.0)) return far;
   }
+  int k;
+  const double r = exp_reduce(x, &k);
+  return exp_finish(r, __dmul_rn(r, r), k);
+}
+
+// exp(x) and exp(-x) for 0 <= x < 704: the reduction is odd in x, so one serves both
+__device__ __forceinline__ void dexp_both(double x, double *up, double *down) {
+  int k;
+  const double r = exp_reduce(x, &k);
+  const double r2 = __dmul_rn(r, r);
+  *up = exp_finish(r, r2, k);
+  *down = exp_finish(-r, r2, -k);
+}
+
+// log of a positive normal x, e0 added to its exponent
+__device__ __forceinline__ double dlog_normal(double x, int e0) {
   unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  e += (int)((b >> 52) & 0x7ff) - 1023;
+  const int e = e0 + (int)((b >> 52) & 0x7ff) - 1023;
   const int j = (int)((b >> 44) & 255);
   b = (b & 0x000fffffffffffffULL) | 0x3ff0000000000000ULL;
   const double m = __longlong_as_double((long long)b);
   const double r = __fma_rn(m, __ldg(&g_log_inv[j]), -1.0);
   // log(1 + r) = r - r^2/2 + r^3/3 - ... - r^6/6
-  double q = -g_mc.inv_fact[3];             // -1/6
-  q = __fma_rn(q, r, g_mc.log_c[2]);        // 1/5
-  q = __fma_rn(q, r, -0.25);
-  q = __fma_rn(q, r, g_mc.log_c[1]);        // 1/3
-  q = __fma_rn(q, r, -0.5);
+  bool exact;
+  double q = log_steps(r, &exact);
+  if (!exact) q = log_steps_any(r);
   const double lp = __fma_rn(q, __dmul_rn(r, r), r);
   const double ed = widen_int((float)e);
   // e kLn2Hi is exact (11 and 29 bits), so the fused sum rounds once, as the separate one
   const double hi = __fma_rn(ed, kLn2Hi, __ldg(&g_log_tab[j]));
   const double lo = __fma_rn(ed, kLn2Lo, lp);
   return __dadd_rn(hi, lo);
+}
+
+// log of anything else
+__device__ __noinline__ double dlog_any(double x) {
+  if (x != x) return x;
+  if (x < 0.0) return __longlong_as_double(0x7ff8000000000000LL);
+  if (x == 0.0) return __longlong_as_double((long long)0xfff0000000000000ULL);
+  if (__double_as_longlong(x) == 0x7ff0000000000000LL) return x;
+  return dlog_normal(__dmul_rn(x, 0x1p54), -54);   // subnormal
+}
+
+__device__ inline double dlog(double x) {
+  const int hx = __double2hiint(x);
+  return hx < 0x00100000 || hx >= 0x7ff00000 ? dlog_any(x) : dlog_normal(x, 0);
 }
 
 __device__ inline double dpow(double x, double y) {
@@ -234,22 +282,23 @@ __device__ inline double dpow(double x, double y) {
 // dpow with the exponent's kind decided ahead: n2 = 2y when y is a positive
 // multiple of 1/2 up to 8 (the case dpow treats with products and a square
 // root), else 0 -- the same results as dpow(x, y) without testing y
-__device__ inline double dpow_n2(double x, double y, int n2) {
-  if (pos(x)) {
-    if (n2 > 0) {
-      const int n = n2 >> 1;
-      double r = 1.0;
-      if (n > 0) {
-        r = x;
-        for (int i = 1; i < n; ++i) r = __dmul_rn(r, x);
-      }
-      if (n2 & 1) r = (n > 0) ? __dmul_rn(r, droot(x)) : droot(x);
-      return r;
-    }
-    return dexp(__dmul_rn(y, dlog(x)));
-  }
+__device__ __noinline__ double dpow_any(double x, double y) {   // x not positive
   if (x == 0.0) return (y > 0.0) ? 0.0 : ((y == 0.0) ? 1.0 : __longlong_as_double(0x7ff0000000000000LL));
   return __longlong_as_double(0x7ff8000000000000LL);
+}
+
+__device__ inline double dpow_n2(double x, double y, int n2) {
+  if (!pos(x)) return dpow_any(x, y);
+  if (n2 == 0) return dexp(__dmul_rn(y, dlog(x)));
+  const int n = n2 >> 1;
+  double r = x;
+#pragma unroll 1
+  for (int i = 1; i < n; ++i) r = __dmul_rn(r, x);
+  if (n2 & 1) {
+    const double root = droot(x);
+    r = n > 0 ? __dmul_rn(r, root) : root;
+  }
+  return r;
 }
 
 // host: n2 of dpow_n2 for a constant exponent

@@ -1,6 +1,6 @@
-"""The integer division and square root of the rate-of-spread path against IEEE-754.
+"""The integer arithmetic of the rate-of-spread path against IEEE-754.
 
-``csrc/c2f_exact.cuh`` compiles as plain C++: both functions must return the
+``csrc/c2f_exact.cuh`` compiles as plain C++: division and square root must return the
 correctly rounded binary64 result (numpy's) over their stated range, for any
 starting estimate within two units of binary32 (the GPU's approximate
 reciprocals are within one).  Arguments sit where the algorithms can go wrong:
@@ -19,6 +19,17 @@ SOURCE = r"""
 static float g_scale = 1.0f;
 #define C2F_HOST_ESTIMATE_SCALE g_scale
 #include "c2f_exact.cuh"
+extern "C" void steps(const double *r, long n, int log, double *q, double *e, unsigned char *ok) {
+  for (long i = 0; i < n; ++i) {
+    bool exact;
+    q[i] = log ? c2f::log_steps(r[i], &exact) : c2f::exp_steps(r[i], &exact);
+    ok[i] = exact;
+    if (log)
+      e[i] = std::fma(std::fma(std::fma(std::fma(-1.0 / 6, r[i], 1.0 / 5), r[i], -0.25), r[i], 1.0 / 3), r[i], -0.5);
+    else
+      e[i] = std::fma(std::fma(std::fma(1.0 / 120, r[i], 1.0 / 24), r[i], 1.0 / 6), r[i], 0.5);
+  }
+}
 extern "C" void run(const double *a, const double *b, long n, int ulps, double *q, double *s, unsigned char *ok) {
   g_scale = 1.0f + ulps * 0x1p-23f;
   for (long i = 0; i < n; ++i) {
@@ -69,3 +80,20 @@ def test_division_and_root_are_correctly_rounded(lib, ulps, span):
     assert use.mean() > 0.99
     assert np.array_equal(q[use], (a / b)[use])
     assert np.array_equal(s[use], np.sqrt(a)[use])
+
+
+def test_exp_and_log_steps_equal_fused_multiply_adds(lib):
+    """Where they say so, the integer Horner steps are the FP64 ones: c + q r rounded at every step."""
+    rng = np.random.default_rng(3)
+    n = 200_000
+    r = rng.uniform(-0.00542, 0.00542, n)
+    r[: n // 4] = np.ldexp(r[: n // 4], -rng.integers(0, 12, n // 4))
+    r[:7] = [0.0, -0.0, 2.0 ** -18, -2.0 ** -18, 2.0 ** -8, -2.0 ** -8, 2.0 ** -40]
+    q, e, ok = np.empty(n), np.empty(n), np.empty(n, dtype=np.uint8)
+    for which in (0, 1):   # exp, log
+        lib.steps(r.ctypes.data_as(C.c_void_p), C.c_long(n), C.c_int(which), q.ctypes.data_as(C.c_void_p),
+                  e.ctypes.data_as(C.c_void_p), ok.ctypes.data_as(C.c_void_p))
+        use = ok.astype(bool)
+        big = np.abs(r) > 2.0 ** -17.9
+        assert use[big & ((r > 0) | (which == 0))].mean() > 0.999
+        assert np.array_equal(q[use], e[use])
