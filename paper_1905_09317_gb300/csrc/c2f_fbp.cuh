@@ -65,15 +65,40 @@ __device__ inline double curing_factor(double c) {
   return __dadd_rn(0.176, __dmul_rn(0.02, __dsub_rn(c, 58.8)));
 }
 
-__device__ inline double rsi_of(int fuel, double isi, double pcf, double cf) {
-  if (fuel == F_M1)
-    return __dadd_rn(__dmul_rn(pcf, rsi_curve(g_fuel[F_C2], isi)),
-                     __dmul_rn(__dsub_rn(1.0, pcf), rsi_curve(g_fuel[F_D1], isi)));
-  if (fuel == F_M2)
-    return __dadd_rn(__dmul_rn(pcf, rsi_curve(g_fuel[F_C2], isi)),
-                     __dmul_rn(0.2, __dmul_rn(__dsub_rn(1.0, pcf), rsi_curve(g_fuel[F_D1], isi))));
-  if (is_o1(fuel)) return __dmul_rn(rsi_curve(g_fuel[fuel], isi), cf);
-  return rsi_curve(g_fuel[fuel], isi);
+// The curves of a fuel: its own, or C2 and D1 for the mixed woods
+__device__ __forceinline__ int curves_of(int fuel) { return fuel == F_M1 || fuel == F_M2 ? 2 : 1; }
+__device__ __forceinline__ int curve_of(int fuel, int i) { return curves_of(fuel) == 1 ? fuel : (i == 0 ? F_C2 : F_D1); }
+
+// RSI at isi[0] and isi[1], in place.  One copy of the curve's code, run twice
+// or (mixed woods) four times: a warp runs the whole of a cell-hour's 3,000
+// instructions from the instruction cache, and with every call inlined a
+// quarter of its stalls were instruction fetches.
+__device__ __forceinline__ void rsi_both(int fuel, double isi[2], double pcf, double cf) {
+  const int nc = curves_of(fuel);
+  double first = 0.0, x = isi[0], other = isi[1], done = 0.0;
+#pragma unroll 1
+  for (int it = 0; it < 2 * nc; ++it) {
+    const int i = nc == 2 ? it & 1 : 0;
+    const double v = rsi_curve(g_fuel[curve_of(fuel, i)], x);
+    if (i + 1 < nc) {
+      first = __dmul_rn(pcf, v);
+      continue;
+    }
+    double r = v;
+    if (nc == 2) {
+      r = __dmul_rn(__dsub_rn(1.0, pcf), v);
+      if (fuel == F_M2) r = __dmul_rn(0.2, r);
+      r = __dadd_rn(first, r);
+    } else if (is_o1(fuel)) {
+      r = __dmul_rn(v, cf);
+    }
+    const double prev = done;   // first round: isi[1] next; second: both results
+    done = r;
+    x = other;
+    other = prev;
+  }
+  isi[0] = other;
+  isi[1] = done;
 }
 
 // ISI at which the (a*mult, b, c) curve gives rsf; the 1 - (rsf/a)^(1/c) term is
@@ -86,21 +111,21 @@ __device__ inline double isf_curve(const FuelCoef &k, double inv_am, double rsf)
   return __dmul_rn(dlog(x), k.neg_inv_b);
 }
 
-__device__ inline double isf_of(int fuel, const HourPrep &hp, double sf, double pcf) {
-  if (fuel == F_M1) {
-    const double rsf_c2 = __dmul_rn(hp.rszf[F_C2], sf);
-    const double rsf_d1 = __dmul_rn(hp.rszf[F_D1], sf);
-    return __dadd_rn(__dmul_rn(pcf, isf_curve(g_fuel[F_C2], hp.inv_a[F_C2], rsf_c2)),
-                     __dmul_rn(__dsub_rn(1.0, pcf), isf_curve(g_fuel[F_D1], hp.inv_a[F_D1], rsf_d1)));
+__device__ __forceinline__ double isf_of(int fuel, const HourPrep &hp, double sf, double pcf) {
+  const int nc = curves_of(fuel);
+  double first = 0.0, r = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < nc; ++i) {   // one copy of the code, as in rsi_both
+    const int f = curve_of(fuel, i);
+    double rsz = hp.rszf[f], inv_am = hp.inv_a[f];
+    if (fuel == F_M2 && i == 1) {
+      rsz = __dmul_rn(0.2, rsz);
+      inv_am = hp.inv_a_d1m2;
+    }
+    r = isf_curve(g_fuel[f], inv_am, __dmul_rn(rsz, sf));
+    if (i + 1 < nc) first = __dmul_rn(pcf, r);
   }
-  if (fuel == F_M2) {
-    const double rsf_c2 = __dmul_rn(hp.rszf[F_C2], sf);
-    const double rsf_d1 = __dmul_rn(__dmul_rn(0.2, hp.rszf[F_D1]), sf);
-    return __dadd_rn(__dmul_rn(pcf, isf_curve(g_fuel[F_C2], hp.inv_a[F_C2], rsf_c2)),
-                     __dmul_rn(__dsub_rn(1.0, pcf), isf_curve(g_fuel[F_D1], hp.inv_a_d1m2, rsf_d1)));
-  }
-  const double rsf = __dmul_rn(hp.rszf[fuel], sf);
-  return isf_curve(g_fuel[fuel], hp.inv_a[fuel], rsf);
+  return nc == 1 ? r : __dadd_rn(first, __dmul_rn(__dsub_rn(1.0, pcf), r));
 }
 
 // wind function of the ISI, up to 40 km/h and in the saturating branch of the 2009 update above,
@@ -215,17 +240,20 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
   if (ellipse_mode == 0) {
     const double e = droot(__dsub_rn(1.0, __dmul_rn(ilb, ilb)));
     const double A = __dmul_rn(a, __dsub_rn(1.0, __dmul_rn(e, e)));
-    const double cph[4] = {ux, dpp, uy, dmp};
     o->back = A;
     o->paired = true;
     o->behind = 0u;
-#pragma unroll
+    double c0 = ux, c1 = dpp, c2 = uy, c3 = dmp, r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;
+#pragma unroll 1
     for (int j = 0; j < 4; ++j) {   // one of the axes j and j + 4 points ahead (neither at cos = 0)
-      const uint64_t c = bits_of(cph[j]);
+      const uint64_t c = bits_of(c0);
       const double ahead = double_of(c & 0x7FFFFFFFFFFFFFFFull);
       o->behind |= (uint32_t)(c >> 63) << j;
-      o->ros[j] = pos(ahead) ? ddiv(A, __dsub_rn(1.0, __dmul_rn(e, ahead))) : A;
+      const double q = pos(ahead) ? ddiv(A, __dsub_rn(1.0, __dmul_rn(e, ahead))) : A;
+      c0 = c1; c1 = c2; c2 = c3;   // the next axis' cosine, in registers
+      r0 = r1; r1 = r2; r2 = r3; r3 = q;
     }
+    o->ros[0] = r0; o->ros[1] = r1; o->ros[2] = r2; o->ros[3] = r3;
   } else {
     // the ray from the ignition point, c = (HROS - BROS)/2 behind the centre,
     // to the ellipse with semi-axes a and b = FROS:
@@ -290,11 +318,10 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
   }
   double fw, fb;
   wind_fn(wsv, &fw, &fb);
-  const double isi = __dmul_rn(hp.isz, fw);
+  double rsi[2] = {__dmul_rn(hp.isz, fw), __dmul_rn(hp.isz, fb)};
+  rsi_both(fuel, rsi, pcf, cf);
   const double be = hp.be[fuel];
-  const double hros = __dmul_rn(rsi_of(fuel, isi, pcf, cf), be);
-  const double bisi = __dmul_rn(hp.isz, fb);
-  const double bros = __dmul_rn(rsi_of(fuel, bisi, pcf, cf), be);
+  const double hros = __dmul_rn(rsi[0], be), bros = __dmul_rn(rsi[1], be);
   double lb;
   if (is_o1(fuel))
     lb = !lt_c(wsv, 1.0) ? __dmul_rn(1.1, dpow_n2(wsv, 0.464, 0)) : 1.0;
