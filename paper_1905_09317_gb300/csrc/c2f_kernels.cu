@@ -333,22 +333,23 @@ __device__ __forceinline__ uint32_t min_byte8(uint64_t v) {
   return min(m & 0xFFFFu, m >> 16);
 }
 
-// The number of periods n <= nmax after which an axis with rem > 0 to go
+// The number of periods n <= nmax <= 60 after which an axis with rem > 0 to go
 // reaches its neighbour's centre at inc a period (the smallest n >= 1 with
-// n * inc >= rem), or 0 if it takes more than nmax <= 60; rem and inc are below
-// 2^(31 + shift).  A binary32 estimate of the quotient from the top bits, never
-// more than its ceiling (inc is rounded up), then one exact int64 step; the
-// estimate falls short by two or more only when inc has few top bits, i.e. for
-// the last few units of a nearly finished axis.
-__device__ __forceinline__ int32_t periods_to_cross(int64_t rem, int64_t inc, int32_t nmax, int shift) {
+// n * inc >= rem), or 0 if it takes more; rem and inc are below 2^(31 + shift).
+// A binary32 estimate of the quotient from the top bits, never more than its
+// ceiling (inc is rounded up), then one exact int64 step.  What is still left
+// after n periods is *left: while it is positive the caller adds one to n and
+// takes inc from it (no branch here, so that callers can work on two axes at a
+// time); that happens only when inc has few top bits, i.e. for the last few
+// units of a nearly finished axis.
+__device__ __forceinline__ int32_t cross_estimate(int64_t rem, int64_t inc, int32_t nmax, int shift, int64_t *left) {
   const bool in_time = inc > 0 && inc * nmax >= rem;
   const float a = (float)(uint32_t)((uint64_t)rem >> shift), b = (float)((uint32_t)((uint64_t)inc >> shift) + 1u);
-  int32_t n = in_time ? (int32_t)__fdividef(a, b) : 0;
-  int64_t left = rem - (int64_t)((uint64_t)(uint32_t)n * (uint64_t)inc);
-  n += left > 0 ? 1 : 0;
-  left -= inc;
-  while (in_time && left > 0) { ++n; left -= inc; }
-  return in_time ? n : 0;
+  const int32_t n = in_time ? (int32_t)__fdividef(a, b) : 0;
+  const int64_t r = rem - (int64_t)((uint64_t)(uint32_t)n * (uint64_t)inc);
+  const int32_t step = in_time && r > 0 ? 1 : 0;
+  *left = in_time ? r - (step ? inc : 0) : 0;
+  return n + step;
 }
 
 // The frontier's two binary64 tests are kept out of line: inlined, the
@@ -438,13 +439,17 @@ __device__ __forceinline__ void table_chunk(const SimJob &J, int32_t h, int32_t 
 // that burned out by it.  With WIN, a window of kWinRows x (32 kWinWords)
 // cells of the Available plane around the ignition cell lives in shared
 // memory and the rest of the grid in global memory; without it, all in global
-// memory.  A cell burned out by A5 (ii) needs no bit of its own: it is one
+// memory.  In global memory the plane holds only the rows [g0, g1) that the
+// fire can reach, or look at, by the end of the hour (reach()); the others are
+// the burnable plane's.  (Copying all of it at the start cost a replica of a
+// 4096 x 4096 landscape 2.7 of its 8.3 ms.)  A cell burned out by A5 (ii) needs no bit of its own: it is one
 // that ignited and has no Available neighbour.
 template <bool WIN>
 struct Planes {
   uint32_t *sav;         // shared-memory window
   uint32_t *gav, *gbr;   // full planes, global memory
-  int32_t r0, w0, rows, wpr;
+  const uint32_t *burnable;
+  int32_t r0, w0, rows, wpr, g0, g1;
   __device__ __forceinline__ bool in_win(int32_t r, int32_t w) const {
     if constexpr (WIN) return (uint32_t)(r - r0) < (uint32_t)kWinRows && (uint32_t)(w - w0) < (uint32_t)kWinWords;
     else return false;
@@ -454,6 +459,38 @@ struct Planes {
     if ((uint32_t)r >= (uint32_t)rows || (uint32_t)w >= (uint32_t)wpr) return 0u;
     if (in_win(r, w)) return sav[(r - r0) * kWinWords + (w - w0)];
     return gav[r * wpr + w];
+  }
+  // copies [i, end) of the burnable plane into the global Available plane
+  // (one warp, eight loads in flight)
+  __device__ __forceinline__ void fill(int32_t i, int32_t end, int lane) const {
+    for (i += lane; i + 7 * 32 < end; i += 8 * 32) {
+      uint32_t v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = __ldg(&burnable[i + 32 * j]);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) gav[i + 32 * j] = v[j];
+    }
+    for (; i < end; i += 32) gav[i] = __ldg(&burnable[i]);
+  }
+  // makes the global rows hold those of rows [ra, rb], columns [ca, cb] and
+  // `far` around them, unless all of that lies in the window (whole warp)
+  __device__ __forceinline__ void reach(int32_t ra, int32_t rb, int32_t ca, int32_t cb, int32_t far, int lane) {
+    ra = max(ra - far, 0);
+    rb = min(rb + far + 1, rows);
+    if constexpr (WIN) {
+      if (ra >= r0 && rb <= r0 + kWinRows && max(ca - far, 0) >> 5 >= w0 && min((cb + far) >> 5, wpr - 1) < w0 + kWinWords)
+        return;   // all in the window
+    }
+    if (g0 == g1) g0 = g1 = ra;   // none yet
+    if (ra < g0) {
+      fill(ra * wpr, g0 * wpr, lane);
+      g0 = ra;
+    }
+    if (rb > g1) {
+      fill(g1 * wpr, rb * wpr, lane);
+      g1 = rb;
+    }
+    __syncwarp();
   }
   // ignition: clears the Available bit
   __device__ __forceinline__ void take(int32_t r, int32_t c) const {
@@ -524,6 +561,11 @@ __device__ __forceinline__ uint32_t bytes_below(uint64_t c8, uint32_t e) {
 
 // a 4-bit mask as bytes: 0xFF where the bit is set
 __device__ __forceinline__ uint32_t bytes_of(uint32_t m) { return ((m & 0xFu) * 0x00204081u & 0x01010101u) * 0xFFu; }
+
+// entries that a window is made long enough for (of the 64 it can hold, by the
+// density of crossings in the last window): about 0.7 crossings an entry lead
+// to Available cells, and a window handles 32
+constexpr int32_t kWindowFill = 36;
 
 // 16 bytes of global memory into shared memory, asynchronously, through L2
 // only (a lazy table's rows may have been written by another SM)
@@ -603,8 +645,9 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   __shared__ __align__(16) int64_t s_prg[WPC][32 * 8];    // hour boundary: their progress
   __shared__ int32_t s_qent[WPC][64];                     // hour boundary: kept entries
   __shared__ uint8_t s_qam[WPC][64];                      // and their open axes
-  __shared__ uint32_t s_buf[WPC][32];                     // a window's entries, crossings, burn-outs
+  __shared__ uint32_t s_buf[WPC][64];                     // a window's entries, crossings, burn-outs
   __shared__ uint8_t s_off[WPC][32];                      // the new cells' offsets
+  __shared__ uint8_t s_items[WPC][256];                   // cell (lane) | axis << 5 items of 32 cells
   __shared__ uint32_t s_dbits[WPC][LAZY ? kWinRows * kWinWords / 32 : 1];   // chunks known done this hour
   __shared__ int32_t s_claim[WPC][LAZY ? 32 : 1];
   __shared__ long long s_prof[WPC][PROF ? kProfCounters : 1];
@@ -612,6 +655,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   int32_t *qent = s_qent[wib];
   uint8_t *qam = s_qam[wib];
   uint32_t *buf = s_buf[wib];
+  uint8_t *ibuf = s_items[wib];
   uint8_t *obuf = s_off[wib];
   uint32_t *dbits = s_dbits[wib];
   int32_t *claim = s_claim[wib];
@@ -663,7 +707,6 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     const float sigma = J.sigma;
     const uint32_t *burnable = J.burnable;
     int32_t *istep = J.ign_step ? J.ign_step + (size_t)r * n : nullptr;
-    const int64_t dk = (k & 1) ? J.d_diag : J.d_orth;   // this lane's axis length
     const int len_shift = max(0, 33 - __clzll(J.d_diag));   // lengths >> len_shift fit 31 bits
     const int32_t ic = J.ign_cell[r];
     // an ignition cell outside the grid or not burnable (possible only for
@@ -680,28 +723,18 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     const int32_t dw0 = min(max((icc >> 5) - kWinWords / 2, 0), max(wpr - kWinWords, 0));
     pl.rows = rows;
     pl.wpr = wpr;
-    bool need_global = true;
+    pl.burnable = burnable;
+    pl.g0 = pl.g1 = 0;
     if constexpr (WIN) {   // window centred on the ignition cell, clamped to the grid
       pl.r0 = min(max(ir - kWinRows / 2, 0), max(rows - kWinRows, 0));
       pl.w0 = min(max((icc >> 5) - kWinWords / 2, 0), max(wpr - kWinWords, 0));
-      need_global = rows > kWinRows || wpr > kWinWords;
 #pragma unroll 8
       for (int32_t i = lane; i < kWinRows * kWinWords; i += 32) {
         const int32_t rr = pl.r0 + i / kWinWords, ww = pl.w0 + i % kWinWords;
         pl.sav[i] = (rr < rows && ww < wpr) ? __ldg(&burnable[rr * wpr + ww]) : 0u;
       }
     }
-    if (need_global) {   // eight loads in flight
-      int32_t i = lane;
-      for (; i + 7 * 32 < pw; i += 8 * 32) {
-        uint32_t v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = __ldg(&burnable[i + 32 * j]);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) pl.gav[i + 32 * j] = v[j];
-      }
-      for (; i < pw; i += 32) pl.gav[i] = __ldg(&burnable[i]);
-    }
+    pl.reach(ir, ir, icc, icc, 2, lane);
     if (use_delta)
       for (int32_t i = lane; i < pw; i += 32) pl.gbr[i] = 0u;
     __syncwarp();
@@ -874,15 +907,18 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       // progress carried to the next; (B4) the entry at its new place.
       {
         int32_t out = 0, queued = 0, b0 = 0;
+        int32_t ra = 0x7fffffff, rb = 0, ca = 0x7fffffff, cb = 0;   // the kept cells' rows and columns
         while (b0 < cnt || queued > 0) {
           if (b0 < cnt && queued < 32) {
             const int32_t e = b0 + lane;
             bool keep = false;
             uint32_t am = 0u;   // open axes toward Available cells
+            int32_t cr = 0, cc = 0;
             if (e < cnt) {
               const uint32_t rc = erc[e];
               const uint32_t m = open_axes(*reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8));
-              const int32_t cr = (int32_t)(rc >> 16), cc = (int32_t)(rc & 0xFFFFu);
+              cr = (int32_t)(rc >> 16);
+              cc = (int32_t)(rc & 0xFFFFu);
               uint32_t b[3];
               pl.template block<1>(cr, cc, b);
               am = m & axes_of_rows(b[0], b[1], b[2]);
@@ -894,6 +930,8 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
               const int32_t at = queued + __popc(bal & lt);
               qent[at] = e;
               qam[at] = (uint8_t)am;
+              ra = min(ra, cr); rb = max(rb, cr);
+              ca = min(ca, cc); cb = max(cb, cc);
             }
             queued += __popc(bal);
             b0 += 32;
@@ -931,36 +969,44 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           // every entry of the batch has been read: its new places (never past
           // its old ones) can be written
           if (act) *reinterpret_cast<uint64_t *>(ecofs + (size_t)(out + lane) * 8) = ~0ull;
-          const uint32_t na = (uint32_t)__popc(am);
-          int32_t at = 0, total = 0;
+          int32_t ni = 0;
+          for (int32_t i0 = 0; i0 < m; i0 += 4) {   // lane k of each 8-lane group looks at axis k of an entry
+            const uint32_t ai = __shfl_sync(FULL, am, (i0 + grp) & 31);   // 0 past the last entry
+            const bool open = (ai >> k) & 1u;
+            const uint32_t bal = __ballot_sync(FULL, open);
+            if (open) ibuf[ni + __popc(bal & lt)] = (uint8_t)((i0 + grp) | (k << 5));
+            ni += __popc(bal);
+          }
+          __syncwarp();
+          for (int32_t t0 = 0; t0 < ni; t0 += 64) {
+            int32_t n2[2], e2[2];
+            int64_t inc2[2], left2[2], P2[2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t bal = __ballot_sync(FULL, (na >> j) & 1u);
-            at += __popc(bal & lt) << j;
-            total += __popc(bal) << j;
-          }
-          for (int32_t t0 = 0; t0 < total; t0 += 32) {
-            while (am != 0u && at < t0 + 32) {
-              const uint32_t q = (uint32_t)(__ffs(am) - 1);
-              am &= am - 1u;
-              buf[at - t0] = (uint32_t)lane | (q << 5);
-              ++at;
+            for (int j = 0; j < 2; ++j) {
+              const int32_t t = t0 + 32 * j + lane;
+              const uint32_t c = t < ni ? ibuf[t] : 0u;
+              const int i = (int)(c & 31u), q = (int)(c >> 5);
+              const float fi = __shfl_sync(FULL, f, i);
+              const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
+              e2[j] = i * 8 + q;
+              inc2[j] = apply_noise(rowbuf[e2[j]], noise_fixed(fi), dq);
+              P2[j] = prgbuf[e2[j]];
+              n2[j] = cross_estimate(dq - P2[j], inc2[j], sph, len_shift, &left2[j]);
+              if (t >= ni) left2[j] = 0;
             }
-            __syncwarp();
-            const bool valid = t0 + lane < total;
-            const uint32_t c = valid ? buf[lane] : 0u;
-            const int i = (int)(c & 31u), q = (int)(c >> 5);
-            const float fi = __shfl_sync(FULL, f, i);
-            const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
-            const int64_t inc = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
-            const int64_t P = prgbuf[i * 8 + q];
-            const int32_t np = periods_to_cross(dq - P, inc, sph, len_shift);
-            if (valid) {
-              ecofs[(size_t)(out + i) * 8 + q] = (uint8_t)(np ? (uint32_t)np - 1u : kOpen);
-              if (!np) eP[(size_t)(out + i) * 8 + q] = P + inc * sph;
+            while (__any_sync(FULL, left2[0] > 0 || left2[1] > 0)) {   // rare
+#pragma unroll
+              for (int j = 0; j < 2; ++j)
+                if (left2[j] > 0) { ++n2[j]; left2[j] -= inc2[j]; }
             }
-            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              if (t0 + 32 * j + lane < ni) {
+                ecofs[(size_t)out * 8 + e2[j]] = (uint8_t)(n2[j] ? (uint32_t)n2[j] - 1u : kOpen);
+                if (!n2[j]) eP[(size_t)out * 8 + e2[j]] = P2[j] + inc2[j] * sph;
+              }
           }
+          __syncwarp();
           uint64_t bit = 0;
           bool burns = false;
           if (act) {
@@ -991,6 +1037,10 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         cnt = out;
         end_list(cnt);
+        // a fire advances by at most one cell a period and looks two cells ahead
+        if (cnt > 0)
+          pl.reach((int32_t)__reduce_min_sync(FULL, (uint32_t)ra), (int32_t)__reduce_max_sync(FULL, (uint32_t)rb),
+                   (int32_t)__reduce_min_sync(FULL, (uint32_t)ca), (int32_t)__reduce_max_sync(FULL, (uint32_t)cb), sph + 2, lane);
         __syncwarp();
       }
       if (prof && lane == 0) pq[1] += clock64() - pc_t;
@@ -1007,7 +1057,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           if (prof && lane == 0) pq[9] += 1;
         }
         const int32_t Ew = min(o1 + width, sph);   // the window is [o1, Ew), shortened below
-        // (A1) the entries that cross in the window, up to 32
+        // (A1) the entries that cross in the window, up to 64
         int32_t got = 0;
         bool full = false;
         for (int32_t g0 = 0; g0 < cnt && !full; g0 += 1024) {
@@ -1018,62 +1068,80 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
             if (g0 + j * 128 >= cnt) break;
             if (e0 < cnt) w |= msb_below(*reinterpret_cast<const uint32_t *>(enx + e0), (uint32_t)Ew) >> j;
           }
-          for (;;) {
-            const uint32_t bal = __ballot_sync(FULL, w != 0u);
-            if (bal == 0u) break;
-            const int32_t pos = got + __popc(bal & lt);
-            if (w && pos < 32) {
-              const int32_t b = 31 - __clz((int)w);
-              w ^= 1u << b;
-              buf[pos] = (uint32_t)(g0 + ((7 - (b & 7)) * 32 + lane) * 4 + (b >> 3));
-            }
-            got += __popc(bal);
-            if (got > 32) { full = true; break; }
+          const uint32_t nw = (uint32_t)__popc(w);   // places by the lanes' counts, a ballot per bit
+          int32_t pos = got;
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            const uint32_t bal = __ballot_sync(FULL, (nw >> j) & 1u);
+            pos += __popc(bal & lt) << j;
+            got += __popc(bal) << j;
           }
+          for (; w != 0u && pos < 64; ++pos) {
+            const int32_t b = 31 - __clz((int)w);
+            w ^= 1u << b;
+            buf[pos] = (uint32_t)(g0 + ((7 - (b & 7)) * 32 + lane) * 4 + (b >> 3));
+          }
+          full = got > 64;
         }
         __syncwarp();
-        if (full && width > 1) { width >>= 1; continue; }   // more than 32: a shorter window
-        got = min(got, 32);
+        if (full && width > 1) {   // more than 64: a shorter window
+          width = max(1, min(width - 1, width * kWindowFill / got));
+          continue;
+        }
+        got = min(got, 64);
         if (prof && lane == 0) pq[8] += clock64() - pc_t;
         if (got == 0) { cal &= ~(1ull << o1); continue; }   // its entries were dropped by a compaction
-        const int32_t ent = lane < got ? (int32_t)buf[lane] : -1;
-        // (A2) the axes that cross in the window, towards Available cells
-        uint64_t cof8 = ~0ull;
-        uint32_t rc = 0u, cand = 0u;
-        if (ent >= 0) {
-          cof8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)ent * 8);
-          rc = erc[ent];
-          cand = bytes_below(cof8, (uint32_t)Ew);
+        // (A2) their crossings in the window towards Available cells: target
+        // cell into buf, offset into obuf; lane l holds entries l and 32 + l
+        int32_t ent[2];
+        uint64_t cof8[2];
+        uint32_t left[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ent[j] = 32 * j + lane < got ? (int32_t)buf[32 * j + lane] : -1;
+        __syncwarp();   // the entries have been read from buf
+        bool broken = false;
+        int32_t np = 0;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          cof8[j] = ~0ull;
+          left[j] = 0u;
+          if (32 * j >= got) continue;
+          uint32_t rc = 0u;
+          if (ent[j] >= 0) {
+            cof8[j] = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)ent[j] * 8);
+            rc = erc[ent[j]];
+            left[j] = bytes_below(cof8[j], (uint32_t)Ew);
+            broken |= left[j] == 0u;
+            uint32_t b[3];
+            pl.template block<1>((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu), b);
+            left[j] &= axes_of_rows(b[0], b[1], b[2]);
+          }
+          while (np < 32) {
+            const uint32_t bal = __ballot_sync(FULL, left[j] != 0u);
+            if (bal == 0u) break;
+            const int32_t pos = np + __popc(bal & lt);
+            if (left[j] && pos < 32) {
+              const int q = __ffs(left[j]) - 1;
+              left[j] &= left[j] - 1u;
+              buf[pos] = rc + (uint32_t)(axis_dr(q) * 65536 + axis_dc(q));
+              obuf[pos] = (uint8_t)__byte_perm((uint32_t)cof8[j], (uint32_t)(cof8[j] >> 32), (uint32_t)q);
+            }
+            np += __popc(bal);
+          }
         }
         // every gathered entry closes an axis, or the hour would not end; cannot happen
-        if (__any_sync(FULL, ent >= 0 && cand == 0u)) { status = 2; break; }
-        if (ent >= 0) {
-          uint32_t b[3];
-          pl.template block<1>((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu), b);
-          cand &= axes_of_rows(b[0], b[1], b[2]);
-        }
-        uint32_t left = cand;
-        int32_t np = 0;   // crossings (entry lane | axis << 5 | offset << 8) into buf
-        while (np < 32) {
-          const uint32_t bal = __ballot_sync(FULL, left != 0u);
-          if (bal == 0u) break;
-          const int32_t pos = np + __popc(bal & lt);
-          if (left && pos < 32) {
-            const uint32_t q = (uint32_t)(__ffs(left) - 1);
-            left &= left - 1u;
-            buf[pos] = (uint32_t)lane | (q << 5) |
-                       ((__byte_perm((uint32_t)cof8, (uint32_t)(cof8 >> 32), q) & 0xFFu) << 8);
-          }
-          np += __popc(bal);
-        }
-        const bool more = __any_sync(FULL, left != 0u);   // more than 32 crossings
+        if (__any_sync(FULL, broken)) { status = 2; break; }
+        const bool more = __any_sync(FULL, (left[0] | left[1]) != 0u);   // more than 32 crossings
         __syncwarp();
-        if (more && width > 1) { width >>= 1; continue; }
+        if (more && width > 1) {
+          width = max(1, min(width - 1, width * 3 / 4));
+          continue;
+        }
         np = min(np, 32);
         // (A3) in the order of their offsets (rank by the offset's bits), one crossing per lane
-        uint32_t pr = lane < np ? buf[lane] : 0u;
+        uint32_t trc = lane < np ? buf[lane] : 0u, toff = lane < np ? obuf[lane] : (uint32_t)o1;
         if (width > 1) {
-          const uint32_t v = (pr >> 8) - (uint32_t)o1;
+          const uint32_t v = toff - (uint32_t)o1;
           uint32_t eq = np >= 32 ? FULL : (1u << np) - 1u;
           int32_t pos = 0;
 #pragma unroll
@@ -1088,13 +1156,17 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           }
           pos += __popc(eq & lt);
           __syncwarp();
-          if (lane < np) buf[pos] = pr;
+          if (lane < np) {
+            buf[pos] = trc;
+            obuf[pos] = (uint8_t)toff;
+          }
           __syncwarp();
-          pr = lane < np ? buf[lane] : 0u;
+          if (lane < np) {
+            trc = buf[lane];
+            toff = obuf[lane];
+          }
         }
-        const uint32_t src = __shfl_sync(FULL, rc, (int)(pr & 31u));
-        const int q = (int)((pr >> 5) & 7u);
-        const int32_t tr = (int32_t)(src >> 16) + axis_dr(q), tc = (int32_t)(src & 0xFFFFu) + axis_dc(q);
+        const int32_t tr = (int32_t)(trc >> 16), tc = (int32_t)(trc & 0xFFFFu);
         bool hit = lane < np;
         if (lazy && !gate_free) {   // the receivers' HROS
           ensure(h, hit, tr, tc);
@@ -1103,20 +1175,20 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         if (!gate_free && hit) hit = receive_ok(J, r, (int64_t)tr * cols + tc, h, n);   // else consumed
         // a cell reached by several crossings ignites at the first of them (row
         // 65535 does not exist, so the idle lanes' keys are no cell)
-        const uint32_t peers = __match_any_sync(FULL, hit ? rc_pack(tr, tc) : (0xFFFF0000u | (uint32_t)lane));
+        const uint32_t peers = __match_any_sync(FULL, hit ? trc : (0xFFFF0000u | (uint32_t)lane));
         const bool won = hit && (peers & lt) == 0u;
         const uint32_t wins = __ballot_sync(FULL, won);
         const int32_t nc = __popc(wins);
         if (won) {
-          buf[__popc(wins & lt)] = rc_pack(tr, tc);
-          obuf[__popc(wins & lt)] = (uint8_t)(pr >> 8);
+          buf[__popc(wins & lt)] = trc;
+          obuf[__popc(wins & lt)] = (uint8_t)toff;
         }
         __syncwarp();
         if (prof && lane == 0) {
           const long long t1 = clock64();
           pq[2] += t1 - pc_t;
           pc_t = t1;
-          pq[10] += 1;
+          pq[10] += got > 32 ? 2 : 1;
         }
         if (cnt + nc > cap) { status = 1; break; }
         // (C1) lane i holds the i-th cell that ignites
@@ -1130,7 +1202,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         float f = 1.0f;
         uint32_t nam = 0u;   // its axes towards Available cells | offset << 8
-        uint32_t fuel9 = 0u; // the burnable cells of the 3 x 3 block around it
+        uint32_t fuel_lo[3] = {0u, 0u, 0u}, fuel_hi[3] = {0u, 0u, 0u};   // the burnable plane around it
         bool dies = false;
         if (act) {
           const int64_t *row = baseh + ncell * 8;
@@ -1143,33 +1215,54 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             const int32_t rr = nr - 1 + d;
-            uint32_t lo = 0u, hi = 0u;
-            if (rr >= 0 && rr < rows) {
-              if (wl >= 0) lo = __ldg(&burnable[rr * wpr + wl]);
-              if (wh < wpr) hi = __ldg(&burnable[rr * wpr + wh]);
-            }
-            fuel9 |= (__funnelshift_r(lo, hi, (uint32_t)(ncol - 1) & 31u) & 7u) << (3 * d);
+            const bool in = rr >= 0 && rr < rows;
+            fuel_lo[d] = in && wl >= 0 ? __ldg(&burnable[rr * wpr + wl]) : 0u;
+            fuel_hi[d] = in && wh < wpr ? __ldg(&burnable[rr * wpr + wh]) : 0u;
           }
           f = noise_factor(seed, (uint32_t)r, (uint32_t)ncell, (uint32_t)h, sigma);
           if (use_delta && below_delta(hrosh, ncell, f, delta)) { dies = true; nam &= ~0xFFu; }   // A5 (i)
         }
         copy_async_wait();
         __syncwarp();
-        // (C2) four cells at a time, lane k of each 8-lane group owning axis k:
-        // first crossings, progress to the end of the hour
-#pragma unroll 2
-        for (int32_t b0 = 0; b0 < nc; b0 += 4) {
-          const int32_t i = b0 + grp;
-          const uint32_t oa = __shfl_sync(FULL, nam, i & 31);
-          const float fi = __shfl_sync(FULL, f, i & 31);
-          const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // nmax: periods left in the hour
-          const int64_t inc = apply_noise(rowbuf[(i & 31) * 8 + k], noise_fixed(fi), dk);
-          const int32_t np = periods_to_cross(dk, inc, nmax, len_shift);
-          const uint32_t cof = ((oa >> k) & 1u) ? (np ? (uint32_t)(o + np) : kOpen) : (uint32_t)kNone;
-          if (i < nc) {
-            ecofs[(size_t)(cnt + i) * 8 + k] = (uint8_t)cof;
-            eP[(size_t)(cnt + i) * 8 + k] = inc * nmax;   // read only while the axis is open
+        // (C2) one open axis per lane, two rounds at a time: first crossings,
+        // progress to the end of the hour
+        if (act) *reinterpret_cast<uint64_t *>(ecofs + (size_t)(cnt + lane) * 8) = ~0ull;
+        int32_t ni = 0;
+        for (int32_t b0 = 0; b0 < nc; b0 += 4) {   // lane k of each 8-lane group looks at axis k of a cell
+          const uint32_t am = __shfl_sync(FULL, nam, (b0 + grp) & 31);   // 0 past the last cell
+          const bool open = (am >> k) & 1u;
+          const uint32_t bal = __ballot_sync(FULL, open);
+          if (open) ibuf[ni + __popc(bal & lt)] = (uint8_t)((b0 + grp) | (k << 5));
+          ni += __popc(bal);
+        }
+        __syncwarp();
+        for (int32_t t0 = 0; t0 < ni; t0 += 64) {
+          int32_t n2[2], e2[2];
+          int64_t inc2[2], left2[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int32_t t = t0 + 32 * j + lane;
+            const uint32_t c = t < ni ? ibuf[t] : 0u;
+            const int i = (int)(c & 31u), q = (int)(c >> 5);
+            const uint32_t oa = __shfl_sync(FULL, nam, i);
+            const float fi = __shfl_sync(FULL, f, i);
+            const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
+            const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // nmax: periods left in the hour
+            inc2[j] = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
+            n2[j] = cross_estimate(dq, inc2[j], nmax, len_shift, &left2[j]);
+            e2[j] = i * 8 + q;
+            if (t < ni) eP[(size_t)cnt * 8 + e2[j]] = inc2[j] * nmax;   // read only while the axis is open
+            e2[j] |= o << 8;
           }
+          while (__any_sync(FULL, left2[0] > 0 || left2[1] > 0)) {   // rare
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+              if (left2[j] > 0) { ++n2[j]; left2[j] -= inc2[j]; }
+          }
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            if (t0 + 32 * j + lane < ni)
+              ecofs[(size_t)cnt * 8 + (e2[j] & 0xFF)] = (uint8_t)(n2[j] ? (e2[j] >> 8) + n2[j] : (int32_t)kOpen);
         }
         __syncwarp();
         // (C3) the window's end, and the cells that ignite before it: taken and listed
@@ -1197,7 +1290,12 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           if (dies && pl.burn(nr, ncol)) out = (1u << 16) + no;
           const uint32_t v0 = b[0] | b[1] | b[2], v1 = b[1] | b[2] | b[3], v2 = b[2] | b[3] | b[4];
           gone = ~((v0 | (v0 >> 1) | (v0 >> 2)) & 7u | (((v1 | (v1 >> 1) | (v1 >> 2)) & 7u) << 3) |
-                   (((v2 | (v2 >> 1) | (v2 >> 2)) & 7u) << 6)) & fuel9;
+                   (((v2 | (v2 >> 1) | (v2 >> 2)) & 7u) << 6));
+          uint32_t fuel9 = 0u;
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+            fuel9 |= (__funnelshift_r(fuel_lo[d], fuel_hi[d], (uint32_t)(ncol - 1) & 31u) & 7u) << (3 * d);
+          gone &= fuel9;
         }
         // A5 (ii): the ignited cells among them have burned out in this window
         // (a cell next to an ignition of the window had an Available neighbour
@@ -1226,17 +1324,13 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
             const uint32_t co = __shfl_sync(FULL, no, (int)(c & 31u));
             const int32_t p = (int32_t)(c >> 5), pr3 = (p * 11) >> 5;   // p / 3
             const int32_t xr = (int32_t)(crc >> 16) + pr3 - 1, xc = (int32_t)(crc & 0xFFFFu) + p - 3 * pr3 - 1;
-            bool first;
-            if (total <= 32) {
-              const uint32_t same = __match_any_sync(FULL, valid ? rc_pack(xr, xc) : (0xFFFF0000u | (uint32_t)lane));
-              first = (same & lt) == 0u;
-            } else {   // no later ignition next to it
-              first = true;
-              for (int32_t j = 0; j < done; ++j) {
-                const uint32_t jrc = __shfl_sync(FULL, nrc, j);
-                if (j > (int32_t)(c & 31u) && abs((int32_t)(jrc >> 16) - xr) <= 1 && abs((int32_t)(jrc & 0xFFFFu) - xc) <= 1)
-                  first = false;
-              }
+            const uint32_t key = valid ? rc_pack(xr, xc) : (0xFFFF0000u | (uint32_t)lane);
+            bool first = (__match_any_sync(FULL, key) & lt) == 0u;
+            if (total > 32) {   // nor in an earlier round (rowbuf is free by now)
+              uint32_t *keys = reinterpret_cast<uint32_t *>(rowbuf);
+              for (int32_t j = 0; j < t0; ++j) first = first && keys[j] != key;
+              __syncwarp();
+              keys[t0 + lane] = key;
             }
             if (valid && first && (!use_delta || pl.burn(xr, xc))) out += (1u << 16) + co;
             __syncwarp();
@@ -1244,18 +1338,22 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         // (C4) the crossings before E are closed
         if (!full) cal &= ~((1ull << E) - 1ull);   // E <= 60
-        const uint64_t old8 = cof8;
-        if (ent >= 0) {
-          uint32_t lo = msb_below((uint32_t)cof8, (uint32_t)E), hi = msb_below((uint32_t)(cof8 >> 32), (uint32_t)E);
+        bool closed[2] = {false, false};
+        uint64_t old8[2] = {cof8[0], cof8[1]};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if (32 * j >= got || ent[j] < 0) continue;
+          uint32_t lo = msb_below((uint32_t)cof8[j], (uint32_t)E), hi = msb_below((uint32_t)(cof8[j] >> 32), (uint32_t)E);
           if (more) {   // crossings that found no lane stay open
-            lo &= ~bytes_of(left);
-            hi &= ~bytes_of(left >> 4);
+            lo &= ~bytes_of(left[j]);
+            hi &= ~bytes_of(left[j] >> 4);
           }
           if (lo | hi) {
-            cof8 = ((uint64_t)((uint32_t)(cof8 >> 32) | (hi >> 7) * 0xFFu) << 32) | ((uint32_t)cof8 | (lo >> 7) * 0xFFu);
-            const uint32_t nx = min_byte8(cof8);
-            *reinterpret_cast<uint64_t *>(ecofs + (size_t)ent * 8) = cof8;
-            enx[ent] = (uint8_t)nx;
+            closed[j] = true;
+            cof8[j] = ((uint64_t)((uint32_t)(cof8[j] >> 32) | (hi >> 7) * 0xFFu) << 32) | ((uint32_t)cof8[j] | (lo >> 7) * 0xFFu);
+            const uint32_t nx = min_byte8(cof8[j]);
+            *reinterpret_cast<uint64_t *>(ecofs + (size_t)ent[j] * 8) = cof8[j];
+            enx[ent[j]] = (uint8_t)nx;
             bits |= cal_bit(nx);
           } else if (more) {
             bits |= 1ull << o1;
@@ -1268,13 +1366,11 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         W += (long long)(burned - done) * s0 + ((int32_t)(ob & 0xFFFFu) - on);
         if (PROF) {
           uint64_t seen = 0;   // periods at which a crossing was processed
-          if (prof && cof8 != old8) {
-            for (int j = 0; j < 8; ++j) {
-              const uint32_t u = (uint32_t)(old8 >> (8 * j)) & 0xFFu;
-              if ((int32_t)u < E) seen |= 1ull << u;
-            }
+          for (int j = 0; j < 16 && prof; ++j) {
+            const uint32_t u = (uint32_t)(old8[j >> 3] >> (8 * (j & 7))) & 0xFFu;
+            if (closed[j >> 3] && (int32_t)u < E) seen |= 1ull << u;
           }
-          const int32_t ch = __popc(__ballot_sync(FULL, cof8 != old8));
+          const int32_t ch = __popc(__ballot_sync(FULL, closed[0])) + __popc(__ballot_sync(FULL, closed[1]));
           seen = cal_or(seen);
           if (prof && lane == 0) {
             pq[3] += clock64() - pc_t;
@@ -1288,8 +1384,9 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         live += done - burned;
         cnt += done;
         end_list(cnt);
-        // the next window: a little longer than what this one reached
-        width = E < Ew ? min(width, E - o1 + 2) : min(2 * width, width_max);
+        // the next window: as long as should fill it, a little longer than what this one reached
+        width = min(max(1, (Ew - o1) * kWindowFill / got), E < Ew ? E - o1 + 2 : width_max);
+        width = min(width, width_max);
         __syncwarp();
         if (live == 0) break;
       }
@@ -1299,17 +1396,27 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       uint32_t *dst = J.ign_plane + (size_t)r * pw;
       auto scar = [&](int32_t i) -> uint32_t {
         const int32_t rr = i / wpr, ww = i - rr * wpr;
-        return __ldg(&burnable[i]) & ~(pl.in_win(rr, ww) ? pl.sav[(rr - pl.r0) * kWinWords + (ww - pl.w0)] : pl.gav[i]);
+        if (pl.in_win(rr, ww)) return __ldg(&burnable[i]) & ~pl.sav[(rr - pl.r0) * kWinWords + (ww - pl.w0)];
+        return rr >= pl.g0 && rr < pl.g1 ? __ldg(&burnable[i]) & ~pl.gav[i] : 0u;
       };
-      int32_t i = lane;
-      for (; i + 3 * 32 < pw; i += 4 * 32) {   // four words in flight
+      // only the rows of the window and of the global plane hold ignited cells
+      int32_t ra = pl.g0, rb = pl.g1;
+      if constexpr (WIN) {
+        ra = pl.g0 == pl.g1 ? pl.r0 : min(pl.r0, pl.g0);
+        rb = pl.g0 == pl.g1 ? min(pl.r0 + kWinRows, rows) : max(min(pl.r0 + kWinRows, rows), pl.g1);
+      }
+      const int32_t ia = ra * wpr, ib = rb * wpr;
+      for (int32_t i = lane; i < ia; i += 32) dst[i] = 0u;
+      for (int32_t i = ib + lane; i < pw; i += 32) dst[i] = 0u;
+      int32_t i = ia + lane;
+      for (; i + 3 * 32 < ib; i += 4 * 32) {   // four words in flight
         uint32_t v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = scar(i + 32 * j);
 #pragma unroll
         for (int j = 0; j < 4; ++j) dst[i + 32 * j] = v[j];
       }
-      for (; i < pw; i += 32) dst[i] = scar(i);
+      for (; i < ib; i += 32) dst[i] = scar(i);
     }
     if (lane == 0) {
       if (A.trace.rec) trace_record(A.trace, kTraceReplica, (uint32_t)r, J.trace_tag, t_start, global_ns());
