@@ -435,6 +435,34 @@ __device__ __forceinline__ void table_chunk(const SimJob &J, int32_t h, int32_t 
   __syncwarp();
 }
 
+// A SIZE x SIZE block of an Available plane from (r, c) on, row by row of SIZE
+// bits, that crosses the window's or the grid's edges or lies outside the
+// window (sav: the window from row r0, word w0 on, or nullptr; cells outside
+// the grid are 0).  Out of line: a warp's path through the frontier is long,
+// and with several warps on a scheduler a fifth of its time went into
+// instruction fetches.
+template <int SIZE>
+__device__ __noinline__ uint32_t block_at_edge(const uint32_t *sav, const uint32_t *gav, int32_t r0, int32_t w0,
+                                               int32_t rows, int32_t wpr, int32_t r, int32_t c) {
+  const int32_t wl = c >> 5, wh = (c + SIZE - 1) >> 5;
+  const bool lo_in = sav != nullptr && (uint32_t)(wl - w0) < (uint32_t)kWinWords;
+  const bool hi_in = sav != nullptr && (uint32_t)(wh - w0) < (uint32_t)kWinWords;
+  uint32_t lo[SIZE], hi[SIZE];
+#pragma unroll
+  for (int d = 0; d < SIZE; ++d) {
+    const int32_t rr = r + d;
+    const bool grid = rr >= 0 && rr < rows, win = (uint32_t)(rr - r0) < (uint32_t)kWinRows;
+    lo[d] = hi[d] = 0u;
+    if (grid && wl >= 0) lo[d] = win && lo_in ? sav[(rr - r0) * kWinWords + (wl - w0)] : gav[rr * wpr + wl];
+    if (grid && wh < wpr) hi[d] = win && hi_in ? sav[(rr - r0) * kWinWords + (wh - w0)] : gav[rr * wpr + wh];
+  }
+  uint32_t v = 0u;
+#pragma unroll
+  for (int d = 0; d < SIZE; ++d)
+    v |= (__funnelshift_r(lo[d], hi[d], (uint32_t)c & 31u) & ((1u << SIZE) - 1u)) << (d * SIZE);
+  return v;
+}
+
 // The replica's Available bit plane, and with A5 (i) on a plane of the cells
 // that burned out by it.  With WIN, a window of kWinRows x (32 kWinWords)
 // cells of the Available plane around the ignition cell lives in shared
@@ -453,12 +481,6 @@ struct Planes {
   __device__ __forceinline__ bool in_win(int32_t r, int32_t w) const {
     if constexpr (WIN) return (uint32_t)(r - r0) < (uint32_t)kWinRows && (uint32_t)(w - w0) < (uint32_t)kWinWords;
     else return false;
-  }
-  // word w of row r of the Available plane (0 outside the grid)
-  __device__ __forceinline__ uint32_t word(int32_t r, int32_t w) const {
-    if ((uint32_t)r >= (uint32_t)rows || (uint32_t)w >= (uint32_t)wpr) return 0u;
-    if (in_win(r, w)) return sav[(r - r0) * kWinWords + (w - w0)];
-    return gav[r * wpr + w];
   }
   // copies [i, end) of the burnable plane into the global Available plane
   // (one warp, eight loads in flight)
@@ -501,25 +523,34 @@ struct Planes {
   }
   // the (2 D + 1) x (2 D + 1) block of Available bits around (r, c), one row
   // per element, bit j = column c - D + j; cells outside the grid are 0.  The
-  // common case lies in the window: a row comes out of two adjacent words by
-  // one funnel shift (bits past the last column and rows past the last one
-  // are 0 there)
+  // common case lies in the window (without one: away from the grid's edges): a
+  // row comes out of two adjacent words by one funnel shift (bits past the last
+  // column and rows past the last one are 0 there)
   template <int D>
   __device__ __forceinline__ void block(int32_t r, int32_t c, uint32_t b[2 * D + 1]) const {
-    const uint32_t sh = (uint32_t)(c - D) & 31u, mask = (1u << (2 * D + 1)) - 1u;
+    constexpr uint32_t mask = (1u << (2 * D + 1)) - 1u;
+    const uint32_t sh = (uint32_t)(c - D) & 31u;
     const int32_t wl = (c - D) >> 5, wh = (c + D) >> 5;
+    const uint32_t *p;
+    int32_t step;
+    bool inside;
     if constexpr (WIN) {
-      if ((uint32_t)(r - D - r0) < (uint32_t)(kWinRows - 2 * D) && wl >= w0 && wh < w0 + kWinWords) {
-        const uint32_t *p = sav + (r - D - r0) * kWinWords - w0;
-#pragma unroll
-        for (int d = 0; d < 2 * D + 1; ++d)
-          b[d] = __funnelshift_r(p[d * kWinWords + wl], p[d * kWinWords + wh], sh) & mask;
-        return;
-      }
+      inside = (uint32_t)(r - D - r0) < (uint32_t)(kWinRows - 2 * D) && wl >= w0 && wh < w0 + kWinWords;
+      p = sav + (r - D - r0) * kWinWords - w0;
+      step = kWinWords;
+    } else {
+      inside = r >= D && r + D < rows && wl >= 0 && wh < wpr;
+      p = gav + (r - D) * wpr;
+      step = wpr;
     }
+    if (inside) {
 #pragma unroll
-    for (int d = 0; d < 2 * D + 1; ++d)
-      b[d] = __funnelshift_r(word(r - D + d, wl), word(r - D + d, wh), sh) & mask;
+      for (int d = 0; d < 2 * D + 1; ++d) b[d] = __funnelshift_r(p[d * step + wl], p[d * step + wh], sh) & mask;
+    } else {
+      const uint32_t v = block_at_edge<2 * D + 1>(WIN ? sav : nullptr, gav, WIN ? r0 : 0, WIN ? w0 : 0, rows, wpr, r - D, c - D);
+#pragma unroll
+      for (int d = 0; d < 2 * D + 1; ++d) b[d] = (v >> (d * (2 * D + 1))) & mask;
+    }
   }
   // A5 (i): has (r, c) burned out by it / the first to mark it so
   __device__ __forceinline__ bool burned(int32_t r, int32_t c) const { return (gbr[r * wpr + (c >> 5)] >> (c & 31)) & 1u; }
@@ -645,7 +676,9 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   __shared__ __align__(16) int64_t s_prg[WPC][32 * 8];    // hour boundary: their progress
   __shared__ int32_t s_qent[WPC][64];                     // hour boundary: kept entries
   __shared__ uint8_t s_qam[WPC][64];                      // and their open axes
-  __shared__ uint32_t s_buf[WPC][64];                     // a window's entries, crossings, burn-outs
+  __shared__ int32_t s_went[WPC][64];                     // a window's entries
+  __shared__ uint8_t s_wleft[WPC][64];                    // and their crossings that found no lane
+  __shared__ uint32_t s_buf[WPC][32];                     // crossings, new cells, burn-outs
   __shared__ uint8_t s_off[WPC][32];                      // the new cells' offsets
   __shared__ uint8_t s_items[WPC][256];                   // cell (lane) | axis << 5 items of 32 cells
   __shared__ uint32_t s_dbits[WPC][LAZY ? kWinRows * kWinWords / 32 : 1];   // chunks known done this hour
@@ -656,6 +689,8 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   uint8_t *qam = s_qam[wib];
   uint32_t *buf = s_buf[wib];
   uint8_t *ibuf = s_items[wib];
+  int32_t *went = s_went[wib];
+  uint8_t *wleft = s_wleft[wib];
   uint8_t *obuf = s_off[wib];
   uint32_t *dbits = s_dbits[wib];
   int32_t *claim = s_claim[wib];
@@ -1079,7 +1114,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           for (; w != 0u && pos < 64; ++pos) {
             const int32_t b = 31 - __clz((int)w);
             w ^= 1u << b;
-            buf[pos] = (uint32_t)(g0 + ((7 - (b & 7)) * 32 + lane) * 4 + (b >> 3));
+            went[pos] = g0 + ((7 - (b & 7)) * 32 + lane) * 4 + (b >> 3);
           }
           full = got > 64;
         }
@@ -1091,47 +1126,41 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         got = min(got, 64);
         if (prof && lane == 0) pq[8] += clock64() - pc_t;
         if (got == 0) { cal &= ~(1ull << o1); continue; }   // its entries were dropped by a compaction
-        // (A2) their crossings in the window towards Available cells: target
-        // cell into buf, offset into obuf; lane l holds entries l and 32 + l
-        int32_t ent[2];
-        uint64_t cof8[2];
-        uint32_t left[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) ent[j] = 32 * j + lane < got ? (int32_t)buf[32 * j + lane] : -1;
-        __syncwarp();   // the entries have been read from buf
-        bool broken = false;
+        // (A2) their crossings in the window towards Available cells, up to
+        // 32: target cell into buf, offset into obuf
+        bool broken = false, more = false;   // more: more than 32 crossings
         int32_t np = 0;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          cof8[j] = ~0ull;
-          left[j] = 0u;
-          if (32 * j >= got) continue;
-          uint32_t rc = 0u;
-          if (ent[j] >= 0) {
-            cof8[j] = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)ent[j] * 8);
-            rc = erc[ent[j]];
-            left[j] = bytes_below(cof8[j], (uint32_t)Ew);
-            broken |= left[j] == 0u;
+#pragma unroll 1
+        for (int32_t i0 = 0; i0 < got; i0 += 32) {
+          uint32_t rc = 0u, left = 0u;
+          uint64_t x8 = ~0ull;
+          if (i0 + lane < got) {
+            const int32_t e = went[i0 + lane];
+            x8 = *reinterpret_cast<const uint64_t *>(ecofs + (size_t)e * 8);
+            rc = erc[e];
+            left = bytes_below(x8, (uint32_t)Ew);
+            broken |= left == 0u;
             uint32_t b[3];
             pl.template block<1>((int32_t)(rc >> 16), (int32_t)(rc & 0xFFFFu), b);
-            left[j] &= axes_of_rows(b[0], b[1], b[2]);
+            left &= axes_of_rows(b[0], b[1], b[2]);
           }
           while (np < 32) {
-            const uint32_t bal = __ballot_sync(FULL, left[j] != 0u);
+            const uint32_t bal = __ballot_sync(FULL, left != 0u);
             if (bal == 0u) break;
             const int32_t pos = np + __popc(bal & lt);
-            if (left[j] && pos < 32) {
-              const int q = __ffs(left[j]) - 1;
-              left[j] &= left[j] - 1u;
+            if (left && pos < 32) {
+              const int q = __ffs(left) - 1;
+              left &= left - 1u;
               buf[pos] = rc + (uint32_t)(axis_dr(q) * 65536 + axis_dc(q));
-              obuf[pos] = (uint8_t)__byte_perm((uint32_t)cof8[j], (uint32_t)(cof8[j] >> 32), (uint32_t)q);
+              obuf[pos] = (uint8_t)__byte_perm((uint32_t)x8, (uint32_t)(x8 >> 32), (uint32_t)q);
             }
             np += __popc(bal);
           }
+          more |= __any_sync(FULL, left != 0u) != 0;
+          wleft[i0 + lane] = (uint8_t)left;
         }
         // every gathered entry closes an axis, or the hour would not end; cannot happen
         if (__any_sync(FULL, broken)) { status = 2; break; }
-        const bool more = __any_sync(FULL, (left[0] | left[1]) != 0u);   // more than 32 crossings
         __syncwarp();
         if (more && width > 1) {
           width = max(1, min(width - 1, width * 3 / 4));
@@ -1338,26 +1367,37 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         // (C4) the crossings before E are closed
         if (!full) cal &= ~((1ull << E) - 1ull);   // E <= 60
-        bool closed[2] = {false, false};
-        uint64_t old8[2] = {cof8[0], cof8[1]};
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          if (32 * j >= got || ent[j] < 0) continue;
-          uint32_t lo = msb_below((uint32_t)cof8[j], (uint32_t)E), hi = msb_below((uint32_t)(cof8[j] >> 32), (uint32_t)E);
-          if (more) {   // crossings that found no lane stay open
-            lo &= ~bytes_of(left[j]);
-            hi &= ~bytes_of(left[j] >> 4);
+        uint64_t seen = 0;      // profile: periods at which a crossing was processed, entries with one
+        int32_t crossed = 0;
+#pragma unroll 1
+        for (int32_t i0 = 0; i0 < got; i0 += 32) {
+          bool closed = false;
+          if (i0 + lane < got) {
+            const int32_t e = went[i0 + lane];
+            uint64_t *at = reinterpret_cast<uint64_t *>(ecofs + (size_t)e * 8);
+            const uint32_t x0 = (uint32_t)*at, x1 = (uint32_t)(*at >> 32);
+            uint32_t lo = msb_below(x0, (uint32_t)E), hi = msb_below(x1, (uint32_t)E);
+            if (more) {   // crossings that found no lane stay open
+              lo &= ~bytes_of(wleft[i0 + lane]);
+              hi &= ~bytes_of(wleft[i0 + lane] >> 4);
+            }
+            closed = (lo | hi) != 0u;
+            if (closed) {
+              const uint64_t v = ((uint64_t)(x1 | (hi >> 7) * 0xFFu) << 32) | (x0 | (lo >> 7) * 0xFFu);
+              const uint32_t nx = min_byte8(v);
+              *at = v;
+              enx[e] = (uint8_t)nx;
+              bits |= cal_bit(nx);
+            } else if (more) {
+              bits |= 1ull << o1;
+            }
+            if (PROF && closed)
+              for (int j = 0; j < 8; ++j) {
+                const uint32_t u = ((j < 4 ? x0 : x1) >> (8 * (j & 3))) & 0xFFu;
+                if ((int32_t)u < E) seen |= 1ull << u;
+              }
           }
-          if (lo | hi) {
-            closed[j] = true;
-            cof8[j] = ((uint64_t)((uint32_t)(cof8[j] >> 32) | (hi >> 7) * 0xFFu) << 32) | ((uint32_t)cof8[j] | (lo >> 7) * 0xFFu);
-            const uint32_t nx = min_byte8(cof8[j]);
-            *reinterpret_cast<uint64_t *>(ecofs + (size_t)ent[j] * 8) = cof8[j];
-            enx[ent[j]] = (uint8_t)nx;
-            bits |= cal_bit(nx);
-          } else if (more) {
-            bits |= 1ull << o1;
-          }
+          if (PROF) crossed += __popc(__ballot_sync(FULL, closed));
         }
         cal |= cal_or(bits);
         const uint32_t ob = __reduce_add_sync(FULL, out);
@@ -1365,17 +1405,11 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         const int32_t burned = (int32_t)(ob >> 16);
         W += (long long)(burned - done) * s0 + ((int32_t)(ob & 0xFFFFu) - on);
         if (PROF) {
-          uint64_t seen = 0;   // periods at which a crossing was processed
-          for (int j = 0; j < 16 && prof; ++j) {
-            const uint32_t u = (uint32_t)(old8[j >> 3] >> (8 * (j & 7))) & 0xFFu;
-            if (closed[j >> 3] && (int32_t)u < E) seen |= 1ull << u;
-          }
-          const int32_t ch = __popc(__ballot_sync(FULL, closed[0])) + __popc(__ballot_sync(FULL, closed[1]));
           seen = cal_or(seen);
           if (prof && lane == 0) {
             pq[3] += clock64() - pc_t;
             if (!full && !more) pq[4] += __popcll(seen);
-            pq[5] += ch;
+            pq[5] += crossed;
             pq[6] += done;
             pq[11] += (done + 3) / 4;
           }
@@ -1438,11 +1472,11 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
 // memory (w), or everything in global memory (g); l: tables filled on demand;
 // p: the per-replica profile counters compiled in (one-warp CTAs; the
 // production kernels leave that code out, which makes them about 4 % faster).
-// Register budgets: one-warp CTAs sized so that 11 fit on an SM (the
-// pipelined steps run the next table build beside the frontier, which more
-// registers a thread would crowd out; fewer would spill); two-warp CTAs so
-// that 5 fit
-__global__ void __launch_bounds__(32, 11) k_frontier_g1(FrontierArgs A) { frontier_warp<1, false, false, false>(A); }
+// Register budgets: one-warp CTAs with windows sized so that 11 fit on an SM
+// (their shared memory allows no more, and fewer registers would spill), those
+// with global lists so that 13 fit (48 waiting requests: 46.1 ms at 11, 43.6 at
+// 13, 43.6 at 16); two-warp CTAs so that 5 fit
+__global__ void __launch_bounds__(32, 13) k_frontier_g1(FrontierArgs A) { frontier_warp<1, false, false, false>(A); }
 __global__ void __launch_bounds__(64, 5) k_frontier_g2(FrontierArgs A) { frontier_warp<2, false, false, false>(A); }
 __global__ void __launch_bounds__(128) k_frontier_g4(FrontierArgs A) { frontier_warp<4, false, false, false>(A); }
 __global__ void __launch_bounds__(32, 11) k_frontier_w1(FrontierArgs A) { frontier_warp<1, true, false, false>(A); }

@@ -698,18 +698,18 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
     const int64_t warps_per_sm =
         attempt == 0 ? (ctx->warps_per_sm > 0 ? (int64_t)ctx->warps_per_sm : std::min<int64_t>(want, 8))
                      : std::min<int64_t>(want, 2);
-    // per CTA: 1 KB reserved by the system and about 5.8 KB of static shared
+    // per CTA: 1 KB reserved by the system and about 6 KB of static shared
     // memory per warp (4 KB of them table rows and progress of 32 cells); with the default sizing, kCoRunSmem per SM is left for
     // kernels that run beside the frontier (the next step's or request's table
     // build, burn counts), whose CTAs could not be placed on a full SM
     const int64_t reserve = (attempt == 0 && ctx->warps_per_sm == 0) ? kCoRunSmem : 0;
     const int64_t per_warp = ((int64_t)ctx->smem_per_sm - reserve - (1024 * warps_per_sm) / wpc -
-                              5800 * warps_per_sm) / warps_per_sm;
+                              6000 * warps_per_sm) / warps_per_sm;
     const int64_t room = (per_warp - (int64_t)kWinRows * kWinWords * 4 - 512) / kEntryBytes;
     win_cap = std::min<int64_t>(cap, std::max<int64_t>(256, room & ~int64_t(63)));
     if (attempt > 0) win_cap = std::max<int64_t>(256, room & ~int64_t(63));
   }
-  const int64_t budget = (int64_t)ctx->smem_optin - 5888 * wpc;
+  const int64_t budget = (int64_t)ctx->smem_optin - 6144 * wpc;
   // (a warp's share is rounded up to 16 bytes: the next warp's lists are read 8 bytes at a time)
   const int64_t win_words = ((int64_t)kWinRows * kWinWords + win_cap * kEntryBytes / 4 + 3) & ~int64_t(3);
   // shared-memory lists only when they hold at least 40 % of the default
