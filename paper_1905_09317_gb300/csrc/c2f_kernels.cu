@@ -337,19 +337,18 @@ __device__ __forceinline__ uint32_t min_byte8(uint64_t v) {
 // reaches its neighbour's centre at inc a period (the smallest n >= 1 with
 // n * inc >= rem), or 0 if it takes more; rem and inc are below 2^(31 + shift).
 // A binary32 estimate of the quotient from the top bits, never more than its
-// ceiling (inc is rounded up), then one exact int64 step.  What is still left
-// after n periods is *left: while it is positive the caller adds one to n and
-// takes inc from it (no branch here, so that callers can work on two axes at a
-// time); that happens only when inc has few top bits, i.e. for the last few
-// units of a nearly finished axis.
-__device__ __forceinline__ int32_t cross_estimate(int64_t rem, int64_t inc, int32_t nmax, int shift, int64_t *left) {
+// ceiling (inc is rounded up), then one exact int64 step; it falls short by two
+// or more only when inc has few top bits, i.e. for the last few units of a
+// nearly finished axis.
+__device__ __forceinline__ int32_t periods_to_cross(int64_t rem, int64_t inc, int32_t nmax, int shift) {
   const bool in_time = inc > 0 && inc * nmax >= rem;
   const float a = (float)(uint32_t)((uint64_t)rem >> shift), b = (float)((uint32_t)((uint64_t)inc >> shift) + 1u);
-  const int32_t n = in_time ? (int32_t)__fdividef(a, b) : 0;
-  const int64_t r = rem - (int64_t)((uint64_t)(uint32_t)n * (uint64_t)inc);
-  const int32_t step = in_time && r > 0 ? 1 : 0;
-  *left = in_time ? r - (step ? inc : 0) : 0;
-  return n + step;
+  int32_t n = in_time ? (int32_t)__fdividef(a, b) : 0;
+  int64_t left = rem - (int64_t)((uint64_t)(uint32_t)n * (uint64_t)inc);
+  n += left > 0 ? 1 : 0;
+  left -= inc;
+  while (in_time && left > 0) { ++n; left -= inc; }
+  return in_time ? n : 0;
 }
 
 // The frontier's two binary64 tests are kept out of line: inlined, the
@@ -596,7 +595,7 @@ __device__ __forceinline__ uint32_t bytes_of(uint32_t m) { return ((m & 0xFu) * 
 // entries that a window is made long enough for (of the 64 it can hold, by the
 // density of crossings in the last window): about 0.7 crossings an entry lead
 // to Available cells, and a window handles 32
-constexpr int32_t kWindowFill = 36;
+constexpr int32_t kWindowFill = 44;
 
 // 16 bytes of global memory into shared memory, asynchronously, through L2
 // only (a lazy table's rows may have been written by another SM)
@@ -1013,33 +1012,20 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
             ni += __popc(bal);
           }
           __syncwarp();
-          for (int32_t t0 = 0; t0 < ni; t0 += 64) {
-            int32_t n2[2], e2[2];
-            int64_t inc2[2], left2[2], P2[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-              const int32_t t = t0 + 32 * j + lane;
-              const uint32_t c = t < ni ? ibuf[t] : 0u;
-              const int i = (int)(c & 31u), q = (int)(c >> 5);
-              const float fi = __shfl_sync(FULL, f, i);
-              const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
-              e2[j] = i * 8 + q;
-              inc2[j] = apply_noise(rowbuf[e2[j]], noise_fixed(fi), dq);
-              P2[j] = prgbuf[e2[j]];
-              n2[j] = cross_estimate(dq - P2[j], inc2[j], sph, len_shift, &left2[j]);
-              if (t >= ni) left2[j] = 0;
+#pragma unroll 1
+          for (int32_t t0 = 0; t0 < ni; t0 += 32) {
+            const bool item = t0 + lane < ni;
+            const uint32_t c = item ? ibuf[t0 + lane] : 0u;
+            const int i = (int)(c & 31u), q = (int)(c >> 5);
+            const float fi = __shfl_sync(FULL, f, i);
+            const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
+            const int64_t inc = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
+            const int64_t P = prgbuf[i * 8 + q];
+            const int32_t n1 = item ? periods_to_cross(dq - P, inc, sph, len_shift) : 0;
+            if (item) {
+              ecofs[(size_t)(out + i) * 8 + q] = (uint8_t)(n1 ? (uint32_t)n1 - 1u : kOpen);
+              if (!n1) eP[(size_t)(out + i) * 8 + q] = P + inc * sph;
             }
-            while (__any_sync(FULL, left2[0] > 0 || left2[1] > 0)) {   // rare
-#pragma unroll
-              for (int j = 0; j < 2; ++j)
-                if (left2[j] > 0) { ++n2[j]; left2[j] -= inc2[j]; }
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-              if (t0 + 32 * j + lane < ni) {
-                ecofs[(size_t)out * 8 + e2[j]] = (uint8_t)(n2[j] ? (uint32_t)n2[j] - 1u : kOpen);
-                if (!n2[j]) eP[(size_t)out * 8 + e2[j]] = P2[j] + inc2[j] * sph;
-              }
           }
           __syncwarp();
           uint64_t bit = 0;
@@ -1097,7 +1083,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         bool full = false;
         for (int32_t g0 = 0; g0 < cnt && !full; g0 += 1024) {
           uint32_t w = 0;   // bit 8 b + 7 - j: byte b of this lane's j-th word crosses
-#pragma unroll
+#pragma unroll 2
           for (int j = 0; j < 8; ++j) {
             const int32_t e0 = g0 + (j * 32 + lane) * 4;
             if (g0 + j * 128 >= cnt) break;
@@ -1173,7 +1159,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           const uint32_t v = toff - (uint32_t)o1;
           uint32_t eq = np >= 32 ? FULL : (1u << np) - 1u;
           int32_t pos = 0;
-#pragma unroll
+#pragma unroll (WIN ? 5 : 1)
           for (int j = 4; j >= 0; --j) {
             const uint32_t bal = __ballot_sync(FULL, (v >> j) & 1u);
             if ((v >> j) & 1u) {
@@ -1253,8 +1239,10 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         copy_async_wait();
         __syncwarp();
-        // (C2) one open axis per lane, two rounds at a time: first crossings,
-        // progress to the end of the hour
+        // (C2) one open axis per lane: first crossings, progress to the end of
+        // the hour.  One round at a time: with two in flight (more code) 4,000
+        // replicas took 5.99 instead of 5.38 ms and 64 no less, for the
+        // instruction fetches
         if (act) *reinterpret_cast<uint64_t *>(ecofs + (size_t)(cnt + lane) * 8) = ~0ull;
         int32_t ni = 0;
         for (int32_t b0 = 0; b0 < nc; b0 += 4) {   // lane k of each 8-lane group looks at axis k of a cell
@@ -1265,33 +1253,21 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
           ni += __popc(bal);
         }
         __syncwarp();
-        for (int32_t t0 = 0; t0 < ni; t0 += 64) {
-          int32_t n2[2], e2[2];
-          int64_t inc2[2], left2[2];
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int32_t t = t0 + 32 * j + lane;
-            const uint32_t c = t < ni ? ibuf[t] : 0u;
-            const int i = (int)(c & 31u), q = (int)(c >> 5);
-            const uint32_t oa = __shfl_sync(FULL, nam, i);
-            const float fi = __shfl_sync(FULL, f, i);
-            const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
-            const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // nmax: periods left in the hour
-            inc2[j] = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
-            n2[j] = cross_estimate(dq, inc2[j], nmax, len_shift, &left2[j]);
-            e2[j] = i * 8 + q;
-            if (t < ni) eP[(size_t)cnt * 8 + e2[j]] = inc2[j] * nmax;   // read only while the axis is open
-            e2[j] |= o << 8;
+#pragma unroll 1
+        for (int32_t t0 = 0; t0 < ni; t0 += 32) {
+          const bool item = t0 + lane < ni;
+          const uint32_t c = item ? ibuf[t0 + lane] : 0u;
+          const int i = (int)(c & 31u), q = (int)(c >> 5);
+          const uint32_t oa = __shfl_sync(FULL, nam, i);
+          const float fi = __shfl_sync(FULL, f, i);
+          const int64_t dq = (q & 1) ? J.d_diag : J.d_orth;
+          const int32_t o = (int32_t)(oa >> 8), nmax = sph - 1 - o;   // nmax: periods left in the hour
+          const int64_t inc = apply_noise(rowbuf[i * 8 + q], noise_fixed(fi), dq);
+          const int32_t n1 = periods_to_cross(dq, inc, nmax, len_shift);
+          if (item) {
+            ecofs[(size_t)(cnt + i) * 8 + q] = (uint8_t)(n1 ? o + n1 : (int32_t)kOpen);
+            eP[(size_t)(cnt + i) * 8 + q] = inc * nmax;   // read only while the axis is open
           }
-          while (__any_sync(FULL, left2[0] > 0 || left2[1] > 0)) {   // rare
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-              if (left2[j] > 0) { ++n2[j]; left2[j] -= inc2[j]; }
-          }
-#pragma unroll
-          for (int j = 0; j < 2; ++j)
-            if (t0 + 32 * j + lane < ni)
-              ecofs[(size_t)cnt * 8 + (e2[j] & 0xFF)] = (uint8_t)(n2[j] ? (e2[j] >> 8) + n2[j] : (int32_t)kOpen);
         }
         __syncwarp();
         // (C3) the window's end, and the cells that ignite before it: taken and listed

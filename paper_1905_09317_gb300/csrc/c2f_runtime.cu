@@ -714,7 +714,12 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
   const int64_t win_words = ((int64_t)kWinRows * kWinWords + win_cap * kEntryBytes / 4 + 3) & ~int64_t(3);
   // shared-memory lists only when they hold at least 40 % of the default
   // capacity: smaller ones overflow on large fires and those replicas run twice
-  const bool use_win = ctx->window_smem && win_words * 4 * wpc <= budget &&
+  // and, unless a sizing is asked for, only when the launch's replicas fit the
+  // SMs at 8 warps each: beyond that the 13 warps an SM that global lists allow
+  // are worth more (512^2 x 2,000 replicas 3.54 ms with shared lists, 3.22 with
+  // global ones; x 1,000, 6.6 warps an SM, 2.28 and 2.63 ms)
+  const bool crowd = attempt == 0 && ctx->warps_per_sm == 0 && todo > 8 * (int64_t)ctx->sm_count;
+  const bool use_win = ctx->window_smem && !crowd && win_words * 4 * wpc <= budget &&
                        (attempt == 0 ? (ctx->warps_per_sm > 0 || 5 * win_cap >= 2 * cap) : win_cap >= cap);
   if (use_win) cap = win_cap;
   const int64_t warp_words = use_win ? win_words : 0;
