@@ -140,51 +140,48 @@ __device__ __forceinline__ void wind_fn(double w, double *ahead, double *back) {
   *back = dexp(-x);
 }
 
-// per weather hour: (ws, wd_from, ffmc, bui) -> HourPrep
-__device__ inline void hour_prep(double ws, double wd_from, double ffmc, double bui, double cf,
-                                 HourPrep *hp) {
+// per weather hour: (ws, wd_from, ffmc, bui) -> HourPrep, by 16 lanes of a
+// half-warp, lane f for fuel code f (each value is computed by one lane with
+// the arithmetic of a single thread; one thread a fuel after the other took
+// some 30 us, half of a small landscape's table)
+__device__ inline void hour_prep(int f, double ws, double wd_from, double ffmc, double bui, double cf, HourPrep *hp) {
   const double m = __ddiv_rn(__dmul_rn(147.2, __dsub_rn(101.0, ffmc)), __dadd_rn(59.5, ffmc));
   const double ff = __dmul_rn(__dmul_rn(91.9, dexp(__dmul_rn(-0.1386, m))),
                               __dadd_rn(1.0, __ddiv_rn(dpow(m, 5.31), 4.93e7)));
-  hp->ws = ws;
-  hp->ff = ff;
-  hp->cf = cf;
-  hp->isz = __dmul_rn(0.208, ff);
-  dsincos_deg(__dadd_rn(wd_from, 180.0), &hp->sin_w, &hp->cos_w);
-  for (int f = 0; f < F_NCODES; ++f) {
-    double be = 1.0;
-    if (f != F_NONE && !is_o1(f)) {
-      const double t = __dmul_rn(50.0, dlog(g_fuel[f].q));
-      const double u = __dsub_rn(__ddiv_rn(1.0, bui), __ddiv_rn(1.0, g_fuel[f].bui0));
-      be = dexp(__dmul_rn(t, u));
-    }
-    hp->be[f] = be;
-    double rz = 0.0;
-    if (f != F_NONE && f != F_M1 && f != F_M2) {
-      rz = rsi_curve(g_fuel[f], hp->isz);
-      if (is_o1(f)) rz = __dmul_rn(rz, cf);
-    }
-    hp->rszf[f] = rz;
-    const double mult = is_o1(f) ? cf : 1.0;
-    hp->inv_a[f] = g_fuel[f].a != 0.0 ? __ddiv_rn(1.0, __dmul_rn(g_fuel[f].a, mult)) : 0.0;
+  const double isz = __dmul_rn(0.208, ff);
+  double be = 1.0;
+  if (f != F_NONE && !is_o1(f)) {
+    const double t = __dmul_rn(50.0, dlog(g_fuel[f].q));
+    const double u = __dsub_rn(__ddiv_rn(1.0, bui), __ddiv_rn(1.0, g_fuel[f].bui0));
+    be = dexp(__dmul_rn(t, u));
   }
-  hp->inv_a_d1m2 = __ddiv_rn(1.0, __dmul_rn(g_fuel[F_D1].a, 0.2));
-  hp->inv_isz = __ddiv_rn(1.0, hp->isz);
-  hp->wsx_w = __dmul_rn(hp->ws, hp->sin_w);
-  hp->wsy_w = __dmul_rn(hp->ws, hp->cos_w);
+  double rz = 0.0;
+  if (f != F_NONE && f != F_M1 && f != F_M2) {
+    rz = rsi_curve(g_fuel[f], isz);
+    if (is_o1(f)) rz = __dmul_rn(rz, cf);
+  }
+  hp->be[f] = be;
+  hp->rszf[f] = rz;
+  hp->inv_a[f] = g_fuel[f].a != 0.0 ? __ddiv_rn(1.0, __dmul_rn(g_fuel[f].a, is_o1(f) ? cf : 1.0)) : 0.0;
   // A lower bound on every fuel's HROS this hour: the RSI curve grows with the
   // ISI and the ISI with the wind (wind_fn >= 1 for w >= 0), so RSI >= RSI at
   // zero wind (rszf); a C2/D1 mixture is at least 0.2 x its smaller part.
-  int32_t pos = 1;
-  for (int f = 1; f < F_NCODES; ++f) {
-    double lo = hp->rszf[f];
-    if (f == F_M1 || f == F_M2) {
-      const double c2 = hp->rszf[F_C2], d1 = hp->rszf[F_D1];
-      lo = __dmul_rn(0.2, c2 < d1 ? c2 : d1);
-    }
-    if (!(__dmul_rn(lo, hp->be[f]) > 1e-150)) pos = 0;
+  const double c2 = __shfl_sync(0xffffffffu, rz, F_C2, 16), d1 = __shfl_sync(0xffffffffu, rz, F_D1, 16);
+  const double lo = f == F_M1 || f == F_M2 ? __dmul_rn(0.2, c2 < d1 ? c2 : d1) : rz;
+  const bool low = f != F_NONE && !(__dmul_rn(lo, be) > 1e-150);
+  const uint32_t any_low = __ballot_sync(0xffffffffu, low) & (0xFFFFu << (threadIdx.x & 16));
+  if (f == 0) {
+    hp->ws = ws;
+    hp->ff = ff;
+    hp->cf = cf;
+    hp->isz = isz;
+    dsincos_deg(__dadd_rn(wd_from, 180.0), &hp->sin_w, &hp->cos_w);
+    hp->inv_a_d1m2 = __ddiv_rn(1.0, __dmul_rn(g_fuel[F_D1].a, 0.2));
+    hp->inv_isz = __ddiv_rn(1.0, isz);
+    hp->wsx_w = __dmul_rn(ws, hp->sin_w);
+    hp->wsy_w = __dmul_rn(ws, hp->cos_w);
+    hp->pos = any_low == 0u ? 1 : 0;
   }
-  hp->pos = pos;
 }
 
 // per cell: slope factor and the upslope direction (aspect is the downslope azimuth)

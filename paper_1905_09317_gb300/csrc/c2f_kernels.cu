@@ -138,14 +138,13 @@ __global__ void k_cell_prep(const float *__restrict__ slope, const float *__rest
   out[i] = cp;
 }
 
-// one thread per hour: weather-only terms
+// 16 threads per hour, one per fuel code: weather-only terms
 __global__ void k_hour_prep(const double *__restrict__ weather, int32_t hours, double o1_curing,
                             HourPrep *out) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= hours) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = min(t >> 4, hours - 1);   // the last block's spare threads repeat the last hour
   const double *w = weather + (size_t)h * 4;
-  const double cf = curing_factor(o1_curing);
-  hour_prep(w[0], w[1], w[2], w[3], cf, &out[h]);
+  hour_prep(t & 15, w[0], w[1], w[2], w[3], curing_factor(o1_curing), &out[h]);
 }
 
 // ------------------------------------------------------------------ K1

@@ -502,7 +502,7 @@ int launch_table(c2f_ctx *ctx, Landscape &L, cudaStream_t st, bool eager) {
   {
     ProfScope prof(ctx, 0, st);
     const int32_t nh = T.n_scen * T.prep_hours;   // every scenario's hours, stacked
-    k_hour_prep<<<grid1(nh, 64), 64, 0, st>>>(T.weather->as<double>(), nh, k.curing,
+    k_hour_prep<<<grid1((int64_t)nh * 16, 64), 64, 0, st>>>(T.weather->as<double>(), nh, k.curing,
                                               T.hour_prep.as<HourPrep>());
     CKL("k_hour_prep");
   }
