@@ -367,7 +367,8 @@ C2F_API int c2f_test_hold_chunk(c2f_ctx *ctx, int32_t landscape_id, int32_t scen
  * and its burning list are staged in shared memory (`smem` != 0, the default)
  * or kept in global memory (0).  With shared memory, smem = 1 sizes each
  * warp's share so that the launch's own replicas are resident at once (up to
- * 8 warps per SM); smem = N in [2, 16] sizes it for N warps per SM, leaving
+ * 8 warps per SM; launches of more than 8 replicas per SM keep them in global
+ * memory, where more warps fit); smem = N in [2, 16] sizes it for N warps per SM, leaving
  * room for frontier launches that run at the same time (serving epochs,
  * pipelined steps).  Results do not depend on any of this; they are tuning
  * knobs.  smem outside [0, 16] is C2F_EINVAL. */
@@ -462,9 +463,10 @@ C2F_API int c2f_trace_count(c2f_ctx *ctx, int64_t *count);
  * 1 cycles at hour boundaries, 2 cycles finding and sending crossings and
  * receiving (A), 3 cycles setting up newly ignited cells (C), 4 fire periods
  * visited, 5 burning cells with a crossing processed, 6 cells ignited,
- * 7 longest burning list, 8 cycles of (A) spent walking the visited period's
- * calendar list, 9 list compactions within an hour, 10 rounds of crossing
- * cells (up to 32 each), 11 new-cell set-up iterations (up to 4 cells each),
+ * 7 longest burning list, 8 cycles of (A) spent finding the burning cells that
+ * cross, 9 list compactions within an hour, 10 rounds of crossing cells (up to
+ * 32 each; a window of periods takes one or two), 11 ignited cells in fours
+ * (rounded up per window),
  * 12-15 zero.  Host memory, n_replicas*16 int64.  C2F_EINVAL if the
  * simulation ran without per-replica counters. */
 C2F_API int c2f_get_replica_profile(c2f_ctx *ctx, int32_t sim_id, int64_t *counters);

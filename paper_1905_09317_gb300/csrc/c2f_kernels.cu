@@ -5,7 +5,7 @@
 //                       axis rates as 2^32 fixed-point per-period increments
 //   k_ignite      (K2)  Step 1 of Alg. 1: ignition cell per replica
 //   k_frontier    (K3)  Step 2 of Alg. 1 for whole replicas: send / receive /
-//                       burn-out per fire period, one CTA per replica
+//                       burn-out in windows of fire periods, one warp per replica
 //   k_burn_prob   (K4)  burn-probability counts over replicas
 //   k_compare_hours / k_compare_final   scar comparison metrics of Sec. 4.1
 // plus landscape set-up (burnable bit plane and list) and result export.
@@ -26,8 +26,8 @@
 // integer function of the progress at the start of the hour; the kernel
 // stores that crossing period (as an offset in the hour) instead of adding
 // the increment every period, and only visits periods at which something
-// happens.  All progress arithmetic is int64, so the crossing periods are the
-// ones the period-by-period loop produces.
+// happens, several of them at a time.  All progress arithmetic is int64, so the
+// crossing periods are the ones the period-by-period loop produces.
 #include <cstdint>
 #include <mutex>
 #include <type_traits>
@@ -625,25 +625,33 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 //   A3  ranked by offset; a cell reached several times ignites at the first;
 //   C1  lane i takes the i-th cell to ignite: table row into shared memory
 //       (asynchronously), perturbation;
-//   C2  four cells at a time, lane k of each 8-lane group owning axis k: the
-//       offsets at which the new cells send, progress to the end of the hour;
+//   C2  one open axis of the new cells per lane: the offset at which it sends,
+//       or its progress to the end of the hour;
 //   C3  E = the earliest of these offsets (at most o1 + width); the cells that
 //       ignite before E are taken and listed (the others stay Available and
 //       their crossings open); cells with no Available neighbour left burn
 //       out at the last ignition next to them;
 //   C4  the crossings before E are closed.
 // Every window is at least one period long (a cell sends after the period in
-// which it ignites).  width follows what the last windows reached.  One period
-// at a time a replica of the 512 x 512 landscape issued about 980 instructions
-// in each of its 1,090 visited periods, most of them in passes that few lanes
-// had work for.
+// which it ignites).  width follows the density of crossings and what the last
+// window reached.
+//
+// What bounds it: a replica is one dependent chain, so with few replicas a
+// warp's instruction count times some five cycles an instruction, and with a
+// dozen warps on an SM the instruction fetches of the long path (hence loops
+// and out-of-line edges rather than unrolled code).  One period at a time, a
+// replica of the 512 x 512 landscape (24 h) issued some 980 instructions in each
+// of its 1,090 visited periods, most of them in passes that few lanes had work
+// for; a window holds 5 to 6 periods there, 25 entries, 18 crossings and 15 new
+// cells.  1,000 replicas: 4.42 ms one period at a time, 2.02 to 2.29 ms now;
+// 64 replicas 1.96 ms.
 template <int WPC, bool WIN, bool LAZY, bool PROF>
 __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
   __shared__ SimJob s_job[WPC];
   constexpr uint32_t FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int k = lane & 7, grp = lane >> 3;   // new-cell set-up: lane k of group grp owns axis k
+  const int k = lane & 7, grp = lane >> 3;   // four cells at a time: lane k of group grp looks at axis k
   const uint32_t lt = (1u << lane) - 1u;
   const size_t slot = (size_t)blockIdx.x * WPC + wib;
   const int32_t cap = A.cap;
@@ -732,10 +740,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
     const bool lazy = LAZY && J.chunk_state != nullptr;
     const double delta = J.delta;
     const bool use_delta = delta > 0.0;   // A5 (i) burn-out on
-    // the longest window (with A5 (i) a cell may stop before its neighbours
-    // are gone, so burn-outs are settled period by period)
-    const int32_t width_max = use_delta ? 1 : 32;
-    int32_t width = use_delta ? 1 : 4;
+    int32_t width = 4;   // of the next window, in periods
     const uint64_t seed = J.seed;
     const float sigma = J.sigma;
     const uint32_t *burnable = J.burnable;
@@ -1303,7 +1308,8 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         }
         // A5 (ii): the ignited cells among them have burned out in this window
         // (a cell next to an ignition of the window had an Available neighbour
-        // before it), at the last ignition next to them
+        // before it), at the last ignition next to them, unless A5 (i) had
+        // them burn out earlier
         if (__any_sync(FULL, gone != 0u)) {
           // the last cells' first: places counted from the highest lane
           const uint32_t ng = (uint32_t)__popc(gone);
@@ -1394,8 +1400,8 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
         cnt += done;
         end_list(cnt);
         // the next window: as long as should fill it, a little longer than what this one reached
-        width = min(max(1, (Ew - o1) * kWindowFill / got), E < Ew ? E - o1 + 2 : width_max);
-        width = min(width, width_max);
+        width = min(max(1, (Ew - o1) * kWindowFill / got), E < Ew ? E - o1 + 2 : 32);
+        width = min(width, 32);
         __syncwarp();
         if (live == 0) break;
       }

@@ -110,7 +110,7 @@ extern "C" C2F_API int c2f_frontier_static(const c2f_frontier_io *io, const c2f_
   const int64_t header = (int64_t)carve(0, 0, 0, R).off_slots;
   const int64_t avail_bytes = (int64_t)kStaticScratchBytes - header - 8 * 256;
   const int64_t fixed_per_slot = pw * 8;          // Available + Burned planes
-  const int64_t per_entry = 4 + 1 + 8 + 64;   // cell, first crossing, crossing offsets, progress
+  const int64_t per_entry = 80;   // 77 bytes (cell, first crossing, crossing offsets, progress), counted as 80
   const int64_t cap_max = std::min<int64_t>(n, (avail_bytes - fixed_per_slot) / per_entry);
   if (cap_max < std::min<int64_t>(n, kStaticMinCap)) return C2F_EINVAL;   // landscape too large
 
