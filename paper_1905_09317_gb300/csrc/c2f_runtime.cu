@@ -157,7 +157,16 @@ struct Sim {
   std::shared_ptr<Table> table;
   int32_t rows = 0, cols = 0, wpr = 0;
   int64_t n = 0;
-  DevBuf ign_plane, ign_step, work, n_ignited, ign_cell, status, scen, prof;
+  DevBuf ign_plane, ign_step, prof;
+  // per replica, one block: work i64, ignited cells, ignition cell, status and,
+  // with weather scenarios, the drawn one (i32 each)
+  DevBuf per;
+  bool has_scen = false;
+  int64_t *work() const { return per.as<int64_t>(); }
+  int32_t *n_ignited() const { return reinterpret_cast<int32_t *>(work() + p.n_replicas); }
+  int32_t *ign_cell() const { return n_ignited() + p.n_replicas; }
+  int32_t *status() const { return ign_cell() + p.n_replicas; }
+  int32_t *scen() const { return has_scen ? status() + p.n_replicas : nullptr; }
   int state = S_PENDING;
   int rc = C2F_OK;
   bool cancel_requested = false;
@@ -171,7 +180,7 @@ struct Sim {
   Sim &operator=(const Sim &) = delete;
   ~Sim() {
     for (auto &r : reads) {
-      for (DevBuf *b : {&ign_plane, &ign_step, &work, &n_ignited, &ign_cell, &status, &scen, &prof})
+      for (DevBuf *b : {&ign_plane, &ign_step, &per, &prof})
         if (b->p) cudaStreamWaitEvent(b->st, r.second, 0);
       cudaEventDestroy(r.second);   // released once recorded work completes
     }
@@ -179,11 +188,11 @@ struct Sim {
 };
 
 struct Scratch {
-  DevBuf ent_cell, ent_next, ent_cofs, ent_P, counter, brn, avail;
+  DevBuf ent_cell, ent_next, ent_cofs, ent_P, brn, avail;
   int64_t slots = 0, cap = 0, brn_words = 0, avail_words = 0;
   void reset() {
     ent_cell.reset(); ent_next.reset(); ent_cofs.reset(); ent_P.reset();
-    counter.reset(); brn.reset(); avail.reset();
+    brn.reset(); avail.reset();
     slots = cap = brn_words = avail_words = 0;
   }
 };
@@ -194,7 +203,12 @@ struct FrontierPlan {
   std::vector<int64_t> begin;
   std::vector<SimJob> jobs;      // host copies stay alive while their uploads are in flight
   std::vector<int64_t> retry;
-  DevBuf djobs, dbegin, dlist;
+  // device block of the plan: jobs, item ranges, the work-list cursor (uploaded as 0)
+  DevBuf dplan, dlist;
+  std::vector<unsigned char> plan_host;
+  SimJob *djobs() const { return dplan.as<SimJob>(); }
+  int64_t *dbegin() const { return reinterpret_cast<int64_t *>(djobs() + sims.size()); }
+  unsigned long long *cursor() const { return reinterpret_cast<unsigned long long *>(dbegin() + sims.size() + 1); }
   int64_t cap = 0, max_n = 0, pw_max = 0, n_items = 0;
   bool lazy = false;   // some simulation's table is filled on demand
   void (*kern)(FrontierArgs) = nullptr;
@@ -235,6 +249,8 @@ struct c2f_ctx {
   int frontier_threads = 32;
   bool window_smem = true;
   int warps_per_sm = 0;        // shared-memory sizing target; 0: this launch's own replicas
+  struct Occupancy { void (*kern)(FrontierArgs); int threads; size_t dyn_smem; int bps; };
+  std::vector<Occupancy> occupancy;   // launch shapes seen (at most 32)
   bool eager_tables = true;   // simulations build their tables with K1 up front
   int64_t cap_override = 0;
   int compact_eighths = 6;     // compaction trigger within an hour: eighths of the list capacity
@@ -571,7 +587,6 @@ int ensure_scratch_once(c2f_ctx *ctx, Scratch &S, cudaStream_t st, int64_t slots
     S.slots = slots;
     S.cap = cap;
   }
-  if (!S.counter.p && (rc = dalloc_on(ctx, S.counter, 64, st))) return rc;
   if (S.slots * pw > S.brn_words) {
     if ((rc = dalloc_on(ctx, S.brn, (size_t)S.slots * pw * 4, st))) return rc;
     S.brn_words = S.slots * pw;
@@ -600,14 +615,9 @@ int alloc_sim(c2f_ctx *ctx, Sim &s, cudaStream_t st) {
     if ((rc = dalloc_on(ctx, s.ign_step, (size_t)L.n * 4 * R, st))) return rc;
     CK(cudaMemsetAsync(s.ign_step.p, 0xFF, (size_t)L.n * 4 * R, st));
   }
-  if ((rc = dalloc_on(ctx, s.work, 8 * R, st))) return rc;
-  if ((rc = dalloc_on(ctx, s.n_ignited, 4 * R, st))) return rc;
-  if ((rc = dalloc_on(ctx, s.ign_cell, 4 * R, st))) return rc;
-  if ((rc = dalloc_on(ctx, s.status, 4 * R, st))) return rc;
-  CK(cudaMemsetAsync(s.status.p, 0, 4 * R, st));
-  if (s.table->n_scen > 1) {
-    if ((rc = dalloc_on(ctx, s.scen, 4 * R, st))) return rc;
-  }
+  s.has_scen = s.table->n_scen > 1;
+  if ((rc = dalloc_on(ctx, s.per, (size_t)(s.has_scen ? 24 : 20) * R, st))) return rc;
+  CK(cudaMemsetAsync(s.status(), 0, 4 * R, st));
   if (ctx->replica_counters) {   // per-replica profile counters of the frontier
     if ((rc = dalloc_on(ctx, s.prof, 8 * kProfCounters * R, st))) return rc;
     CK(cudaMemsetAsync(s.prof.p, 0, 8 * kProfCounters * R, st));
@@ -642,7 +652,7 @@ SimJob job_of(const Sim &s) {
   j.scen_thr = T.n_scen > 1
       ? reinterpret_cast<const uint64_t *>(T.weather->as<double>() + (size_t)T.n_scen * T.prep_hours * 4)
       : nullptr;
-  j.scen = s.scen.as<int32_t>();
+  j.scen = s.scen();
   j.seed = s.p.seed;
   j.sigma = (float)s.p.ros_sigma;
   j.ignition_mode = s.p.ignition_mode;
@@ -659,10 +669,10 @@ SimJob job_of(const Sim &s) {
   j.n_replicas = s.p.n_replicas;
   j.ign_plane = s.ign_plane.as<uint32_t>();
   j.ign_step = s.ign_step.as<int32_t>();
-  j.work = s.work.as<int64_t>();
-  j.n_ignited = s.n_ignited.as<int32_t>();
-  j.ign_cell = s.ign_cell.as<int32_t>();
-  j.status = s.status.as<int32_t>();
+  j.work = s.work();
+  j.n_ignited = s.n_ignited();
+  j.ign_cell = s.ign_cell();
+  j.status = s.status();
   j.prof = s.prof.as<long long>();
   j.trace_tag = s.serial;
   return j;
@@ -730,27 +740,33 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
     F.kern = F.lazy ? (use_win ? k_frontier_plw1 : k_frontier_plg1) : (use_win ? k_frontier_pw1 : k_frontier_pg1);
   F.dyn_smem = (size_t)warp_words * 4 * wpc;
   F.threads = threads;
-  if (F.dyn_smem > 0) {   // only ever raised: plans made earlier may still be launched
-    cudaFuncAttributes fa{};
-    CK(cudaFuncGetAttributes(&fa, F.kern));
-    if ((int)F.dyn_smem > fa.maxDynamicSharedSizeBytes)
-      CK(cudaFuncSetAttribute(F.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.dyn_smem));
-  }
   int bps = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, F.kern, threads, F.dyn_smem));
-  bps = std::max(bps, 1);
+  for (const auto &o : ctx->occupancy)   // a pure function of the device, asked for once per shape
+    if (o.kern == F.kern && o.threads == threads && o.dyn_smem == F.dyn_smem) bps = o.bps;
+  if (bps == 0) {
+    if (F.dyn_smem > 0) {   // only ever raised: plans made earlier may still be launched
+      cudaFuncAttributes fa{};
+      CK(cudaFuncGetAttributes(&fa, F.kern));
+      if ((int)F.dyn_smem > fa.maxDynamicSharedSizeBytes)
+        CK(cudaFuncSetAttribute(F.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.dyn_smem));
+    }
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, F.kern, threads, F.dyn_smem));
+    bps = std::max(bps, 1);
+    if (ctx->occupancy.size() >= 32) ctx->occupancy.erase(ctx->occupancy.begin());
+    ctx->occupancy.push_back({F.kern, threads, F.dyn_smem, bps});
+  }
   const int64_t max_ctas = (int64_t)ctx->sm_count * bps;
   F.ctas = std::min<int64_t>((todo + wpc - 1) / wpc, max_ctas);
   const int64_t slots = F.ctas * wpc;   // one warp per slot
   if ((rc = ensure_scratch(ctx, S, st, slots, cap, F.pw_max))) return rc;
   FrontierArgs &A = F.A;
   A = FrontierArgs{};
-  A.jobs = F.djobs.as<SimJob>();
+  A.jobs = F.djobs();
   A.n_jobs = (int32_t)F.sims.size();
-  A.item_begin = F.dbegin.as<int64_t>();
+  A.item_begin = F.dbegin();
   A.item_list = nullptr;
   A.n_items = todo;
-  A.counter = S.counter.as<unsigned long long>();
+  A.counter = F.cursor();
   A.cap = (int32_t)cap;
   A.ent_cell = S.ent_cell.as<int32_t>();
   A.ent_next = S.ent_next.as<uint8_t>();
@@ -793,22 +809,23 @@ int plan_frontier(c2f_ctx *ctx, const std::vector<Sim *> &sims, FrontierPlan &F,
   }
   F.n_items = F.begin[nj];
   int rc;
-  if ((rc = dalloc_on(ctx, F.djobs, sizeof(SimJob) * nj, st))) return rc;
-  if ((rc = dalloc_on(ctx, F.dbegin, sizeof(int64_t) * (nj + 1), st))) return rc;
-  CK(cudaMemcpyAsync(F.djobs.p, jobs.data(), sizeof(SimJob) * nj, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(F.dbegin.p, F.begin.data(), sizeof(int64_t) * (nj + 1), cudaMemcpyHostToDevice, st));
+  const size_t jb = sizeof(SimJob) * (size_t)nj, bb = sizeof(int64_t) * (size_t)(nj + 1);
+  F.plan_host.assign(jb + bb + 8, 0);
+  std::memcpy(F.plan_host.data(), jobs.data(), jb);
+  std::memcpy(F.plan_host.data() + jb, F.begin.data(), bb);
+  if ((rc = dalloc_on(ctx, F.dplan, F.plan_host.size(), st))) return rc;
+  CK(cudaMemcpyAsync(F.dplan.p, F.plan_host.data(), F.plan_host.size(), cudaMemcpyHostToDevice, st));
   return shape_frontier(ctx, F, S, st, F.n_items, F.cap, 0);
 }
 
-int launch_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st) {
+int launch_frontier(c2f_ctx *ctx, FrontierPlan &F, cudaStream_t st) {
   {
     ProfScope prof(ctx, 1, st);
     for (size_t i = 0; i < F.sims.size(); ++i) {
-      k_ignite<<<grid1(F.sims[i]->p.n_replicas, 128), 128, 0, st>>>(F.djobs.as<SimJob>(), (int32_t)i);
+      k_ignite<<<grid1(F.sims[i]->p.n_replicas, 128), 128, 0, st>>>(F.djobs(), (int32_t)i);
       CKL("k_ignite");
     }
   }
-  CK(cudaMemsetAsync(S.counter.p, 0, 8, st));
   ProfScope prof(ctx, 2, st);
   F.kern<<<(unsigned)F.ctas, F.threads, F.dyn_smem, st>>>(F.A);
   CKL("k_frontier");
@@ -823,7 +840,7 @@ int finish_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st) 
     for (int32_t i = 0; i < nj; ++i) {
       const int32_t R = F.sims[i]->p.n_replicas;
       std::vector<int32_t> stv(R);
-      CK(cudaMemcpyAsync(stv.data(), F.sims[i]->status.p, 4 * (size_t)R, cudaMemcpyDeviceToHost, st));
+      CK(cudaMemcpyAsync(stv.data(), F.sims[i]->status(), 4 * (size_t)R, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
       for (int32_t r = 0; r < R; ++r) {
         if (stv[r] == 4)
@@ -840,7 +857,7 @@ int finish_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st) 
       const int32_t i = (int32_t)(std::upper_bound(F.begin.begin(), F.begin.end(), it) - F.begin.begin() - 1);
       const int64_t r = it - F.begin[i];
       Sim &s = *F.sims[i];
-      CK(cudaMemsetAsync(s.status.as<int32_t>() + r, 0, 4, st));
+      CK(cudaMemsetAsync(s.status() + r, 0, 4, st));
       if (s.ign_step.p)
         CK(cudaMemsetAsync(s.ign_step.as<int32_t>() + r * s.n, 0xFF, (size_t)s.n * 4, st));
     }
@@ -849,7 +866,7 @@ int finish_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st) 
     if ((rc = dalloc_on(ctx, F.dlist, sizeof(int64_t) * F.retry.size(), st))) return rc;
     CK(cudaMemcpyAsync(F.dlist.p, F.retry.data(), sizeof(int64_t) * F.retry.size(), cudaMemcpyHostToDevice, st));
     F.A.item_list = F.dlist.as<int64_t>();
-    CK(cudaMemsetAsync(S.counter.p, 0, 8, st));
+    CK(cudaMemsetAsync(F.cursor(), 0, 8, st));
     {
       ProfScope prof(ctx, 2, st);
       F.kern<<<(unsigned)F.ctas, F.threads, F.dyn_smem, st>>>(F.A);
@@ -998,7 +1015,7 @@ int simulate_many(c2f_ctx *ctx, int32_t n, const int32_t *ids, const c2f_sim_par
         if (e == cudaSuccess) e = cudaStreamWaitEvent(gst[g], fork, 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "fork");
       }
-      lrc = launch_frontier(ctx, F[g], scratch_of(g), gst[g]);
+      lrc = launch_frontier(ctx, F[g], gst[g]);
       if (!lrc && gst[g] != ctx->stream) {
         cudaEvent_t join;
         cudaError_t e = new_event(&join);
@@ -1095,7 +1112,7 @@ int reap(c2f_ctx *ctx, bool block) {
     if (rc && !first_rc) first_rc = rc;
     cudaStreamSynchronize(E.stream);
     cudaEventDestroy(E.done);
-    E.F.djobs.reset(); E.F.dbegin.reset(); E.F.dlist.reset();
+    E.F.dplan.reset(); E.F.dlist.reset();
     E.scratch.reset();
     cudaStreamSynchronize(E.stream);   // the scratch frees above are ordered on it
     ctx->stream_pool.push_back(E.stream);
@@ -1145,7 +1162,7 @@ int launch_pending(c2f_ctx *ctx) {
     if (!rc) rc = alloc_sim(ctx, *s, E->stream);
   }
   if (!rc) rc = plan_frontier(ctx, raw, E->F, E->scratch, E->stream);
-  if (!rc) rc = launch_frontier(ctx, E->F, E->scratch, E->stream);
+  if (!rc) rc = launch_frontier(ctx, E->F, E->stream);
   if (rc) {
     for (auto &s : batch) { s->state = S_FAILED; s->rc = rc; }
     cudaStreamSynchronize(E->stream);
@@ -1653,7 +1670,7 @@ C2F_API int c2f_burn_prob_scenario(c2f_ctx *ctx, int32_t sim_id, int32_t scenari
   cudaStream_t st = ctx->read_stream;
   DevBuf tmp;
   if ((rc = dalloc_on(ctx, tmp, (size_t)s->n * 4, st))) return rc;
-  if ((rc = burn_prob_into(ctx, *s, tmp.as<uint32_t>(), st, s->scen.as<int32_t>(), scenario))) return rc;
+  if ((rc = burn_prob_into(ctx, *s, tmp.as<uint32_t>(), st, s->scen(), scenario))) return rc;
   CK(cudaMemcpyAsync(counts, tmp.p, (size_t)s->n * 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return C2F_OK;
@@ -1854,10 +1871,14 @@ C2F_API int c2f_get_counters(c2f_ctx *ctx, int32_t sim_id, int64_t *work, int32_
   CK(cudaSetDevice(ctx->device));
   const size_t R = (size_t)s->p.n_replicas;
   cudaStream_t st = ctx->read_stream;
-  if (work) CK(cudaMemcpyAsync(work, s->work.p, R * 8, cudaMemcpyDeviceToHost, st));
-  if (ignited) CK(cudaMemcpyAsync(ignited, s->n_ignited.p, R * 4, cudaMemcpyDeviceToHost, st));
-  if (ign_cell) CK(cudaMemcpyAsync(ign_cell, s->ign_cell.p, R * 4, cudaMemcpyDeviceToHost, st));
+  // one read of the block that holds them all (a copy to pageable memory waits
+  // for the device, so three in a row cost three round trips)
+  std::vector<unsigned char> host(R * 16);
+  CK(cudaMemcpyAsync(host.data(), s->per.p, host.size(), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (work) std::memcpy(work, host.data(), R * 8);
+  if (ignited) std::memcpy(ignited, host.data() + R * 8, R * 4);
+  if (ign_cell) std::memcpy(ign_cell, host.data() + R * 12, R * 4);
   return C2F_OK;
 }
 
@@ -1870,13 +1891,13 @@ C2F_API int c2f_get_scenarios(c2f_ctx *ctx, int32_t sim_id, int32_t *scenario) {
   int rc = sim_ready(ctx, *s);
   if (rc) return rc;
   const size_t R = (size_t)s->p.n_replicas;
-  if (!s->scen.p) {   // one weather stream: every replica ran scenario 0
+  if (!s->has_scen) {   // one weather stream: every replica ran scenario 0
     std::memset(scenario, 0, R * 4);
     return C2F_OK;
   }
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->read_stream;
-  CK(cudaMemcpyAsync(scenario, s->scen.p, R * 4, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(scenario, s->scen(), R * 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return C2F_OK;
 }
