@@ -604,6 +604,29 @@ __device__ __forceinline__ void copy_async16(void *dst, const void *src) {
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Chunks of on-demand table rows that a frontier warp hands to its CTA's
+// helper warps: n chunks of hour h of job *job (n < 0: no more will come).
+struct ChunkWork {
+  const SimJob *job;
+  int32_t h, n, chunk[32];
+};
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// a helper warp (wib = 1 .. helpers): waits at barrier 1 for chunks, computes
+// every (helpers + 1)-th of them from its own number on, meets at barrier 2
+template <int HELPERS>
+__device__ __forceinline__ void help_with_chunks(const ChunkWork *work) {
+  constexpr int kThreads = 32 * (HELPERS + 1);
+  for (;;) {
+    bar_sync(1, kThreads);
+    const int32_t n = work->n;
+    if (n < 0) return;
+    for (int32_t i = threadIdx.x >> 5; i < n; i += HELPERS + 1) table_chunk(*work->job, work->h, work->chunk[i]);
+    bar_sync(2, kThreads);
+  }
+}
+
 // One warp per replica; replicas come from a work list of (simulation,
 // replica) items that every warp pulls from.  There is no CTA barrier: the
 // warp's counters stay in registers, appends to the burning list are placed
@@ -645,8 +668,11 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 // for; a window holds 5 to 6 periods there, 25 entries, 18 crossings and 15 new
 // cells.  1,000 replicas: 4.42 ms one period at a time, 2.02 to 2.29 ms now;
 // 64 replicas 1.96 ms.
-template <int WPC, bool WIN, bool LAZY, bool PROF>
-__device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
+//
+// HELPERS warps of the CTA beside the frontier's own only compute on-demand
+// table rows (with WPC = 1; `work` in shared memory).
+template <int WPC, bool WIN, bool LAZY, bool PROF, int HELPERS = 0>
+__device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *work = nullptr) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
   __shared__ SimJob s_job[WPC];
   constexpr uint32_t FULL = 0xffffffffu;
@@ -699,7 +725,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
   uint8_t *wleft = s_wleft[wib];
   uint8_t *obuf = s_off[wib];
   uint32_t *dbits = s_dbits[wib];
-  int32_t *claim = s_claim[wib];
+  int32_t *claim = HELPERS > 0 ? work->chunk : s_claim[wib];
   SimJob &J = s_job[wib];
 
   for (;;) {
@@ -843,7 +869,23 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A) {
       if (mine) claim[__popc(mb & lt)] = w;
       __syncwarp();
       const int nm = __popc(mb);
-      for (int i = 0; i < nm; ++i) table_chunk(J, h, claim[i]);
+      if constexpr (HELPERS > 0) {
+        if (nm > 1) {
+          if (lane == 0) {
+            work->job = &J;
+            work->h = h;
+            work->n = nm;
+          }
+          __syncwarp();
+          bar_sync(1, 32 * (HELPERS + 1));
+          for (int i = 0; i < nm; i += HELPERS + 1) table_chunk(J, h, claim[i]);
+          bar_sync(2, 32 * (HELPERS + 1));
+        } else if (nm == 1) {
+          table_chunk(J, h, claim[0]);
+        }
+      } else {
+        for (int i = 0; i < nm; ++i) table_chunk(J, h, claim[i]);
+      }
       if (mine && inwin) atomicOr(&dbits[bi >> 5], 1u << (bi & 31));
       if (need) {
         uint32_t polls = 0;
@@ -1469,6 +1511,24 @@ __global__ void __launch_bounds__(32, 11) k_frontier_pw1(FrontierArgs A) { front
 // frontier needs the whole register budget of a one-warp CTA
 __global__ void __launch_bounds__(32, 1) k_frontier_lg1(FrontierArgs A) { frontier_warp<1, false, true, false>(A); }
 __global__ void __launch_bounds__(32, 1) k_frontier_lw1(FrontierArgs A) { frontier_warp<1, true, true, false>(A); }
+// the same with seven helper warps, for launches that leave SMs to spare: a
+// single warp computes 32 rows at the FP64 unit's latency (few fires on
+// 4096 x 4096, 8 replicas: three quarters of their time)
+constexpr int kHelpers = 7;
+template <bool WIN>
+__device__ __forceinline__ void frontier_helped(const FrontierArgs &A) {
+  __shared__ ChunkWork work;
+  if (threadIdx.x >= 32) {
+    help_with_chunks<kHelpers>(&work);
+    return;
+  }
+  frontier_warp<1, WIN, true, false, kHelpers>(A, &work);
+  if (threadIdx.x == 0) work.n = -1;
+  __syncwarp();
+  bar_sync(1, 32 * (kHelpers + 1));
+}
+__global__ void __launch_bounds__(32 * (kHelpers + 1), 1) k_frontier_lg1h(FrontierArgs A) { frontier_helped<false>(A); }
+__global__ void __launch_bounds__(32 * (kHelpers + 1), 1) k_frontier_lw1h(FrontierArgs A) { frontier_helped<true>(A); }
 __global__ void __launch_bounds__(32, 1) k_frontier_plg1(FrontierArgs A) { frontier_warp<1, false, true, true>(A); }
 __global__ void __launch_bounds__(32, 1) k_frontier_plw1(FrontierArgs A) { frontier_warp<1, true, true, true>(A); }
 

@@ -62,6 +62,8 @@ __global__ void k_frontier_w2(FrontierArgs);
 __global__ void k_frontier_w4(FrontierArgs);
 __global__ void k_frontier_lg1(FrontierArgs);
 __global__ void k_frontier_lw1(FrontierArgs);
+__global__ void k_frontier_lg1h(FrontierArgs);
+__global__ void k_frontier_lw1h(FrontierArgs);
 __global__ void k_frontier_pg1(FrontierArgs);
 __global__ void k_frontier_pw1(FrontierArgs);
 __global__ void k_frontier_plg1(FrontierArgs);
@@ -699,8 +701,13 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
   int rc;
   // 32, 64 or 128: one replica per warp; the profiling kernels (per-replica
   // counters) are one-warp CTAs
-  const int threads = (F.lazy || ctx->replica_counters) ? 32 : ctx->frontier_threads;
-  const int wpc = threads / 32;
+  // on-demand tables: CTAs of one frontier warp, with seven helper warps (one
+  // such CTA an SM) up to two waves of replicas; more replicas keep the SMs busy
+  // by themselves, eight warps each (2048 x 2048 x 48 h: 152 replicas 16 ms with
+  // helpers, 160 without 41 ms, 400 without 49 ms)
+  const bool helped = F.lazy && !ctx->replica_counters && todo <= 2 * (int64_t)ctx->sm_count;
+  const int wpc = (F.lazy || ctx->replica_counters) ? 1 : ctx->frontier_threads / 32;
+  const int threads = helped ? 256 : 32 * wpc;
   int64_t cap = (cap_in + 3) & ~int64_t(3);
   int64_t win_cap = cap;
   {
@@ -735,7 +742,7 @@ int shape_frontier(c2f_ctx *ctx, FrontierPlan &F, Scratch &S, cudaStream_t st, i
   const int64_t warp_words = use_win ? win_words : 0;
   F.kern = use_win ? (wpc == 1 ? k_frontier_w1 : wpc == 2 ? k_frontier_w2 : k_frontier_w4)
                    : (wpc == 1 ? k_frontier_g1 : wpc == 2 ? k_frontier_g2 : k_frontier_g4);
-  if (F.lazy) F.kern = use_win ? k_frontier_lw1 : k_frontier_lg1;
+  if (F.lazy) F.kern = use_win ? (helped ? k_frontier_lw1h : k_frontier_lw1) : (helped ? k_frontier_lg1h : k_frontier_lg1);
   if (ctx->replica_counters)
     F.kern = F.lazy ? (use_win ? k_frontier_plw1 : k_frontier_plg1) : (use_win ? k_frontier_pw1 : k_frontier_pg1);
   F.dyn_smem = (size_t)warp_words * 4 * wpc;

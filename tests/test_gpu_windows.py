@@ -108,3 +108,54 @@ def test_rates_at_the_ends_of_the_range(ctx, ellipse_mode, minutes):
             assert hros[c] == hr, (h, c)
     o.close()
     ctx.release(lid)
+
+
+@pytest.mark.parametrize("replicas", [1, 5, 320])
+@pytest.mark.parametrize("smem", [1, 0])
+def test_helped_on_demand_rows_equal_the_eager_table(ctx, smem, replicas):
+    """On-demand tables: one replica, a few, and more than two an SM (no helper warps); a window of new
+    chunks from one to thirty-two at a time."""
+    w = S.config2(side=301, n_replicas=replicas, hours=6)
+    L = w.landscape
+    p = _params(dict(w.params, ros_threshold=1.0))
+    ctx.set_frontier_config(32, smem)
+    out = []
+    try:
+        for eager in (False, True):
+            ctx.set_table_mode(eager)
+            lid = ctx.load_landscape(L.fuel, L.slope, L.aspect, cell_size=L.cell_size)
+            ctx.set_weather(lid, w.weather)
+            sid = ctx.simulate(lid, p)
+            out.append((ctx.get_counters(sid, replicas), ctx.burn_prob(sid, L.fuel.size),
+                        ctx.get_replica_scar(sid, replicas - 1, L.fuel.size, ign_steps=True)))
+            ctx.release(sid)
+            ctx.release(lid)
+    finally:
+        ctx.set_frontier_config(32, 1)
+        ctx.set_table_mode(True)
+    for a, b in zip(out[0][0], out[1][0]):
+        assert np.array_equal(a, b)
+    assert np.array_equal(out[0][1], out[1][1])
+    for a, b in zip(out[0][2], out[1][2]):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("replicas", [1215, 1217, 2500])
+def test_crowded_launches_equal_small_ones(ctx, replicas):
+    """Above eight replicas an SM the frontier takes global lists: the same replicas, alone and in the crowd."""
+    w = S.config2(side=90, n_replicas=replicas, hours=5)
+    L = w.landscape
+    lid = ctx.load_landscape(L.fuel, L.slope, L.aspect, cell_size=L.cell_size)
+    ctx.set_weather(lid, w.weather)
+    n = L.fuel.size
+    sid = ctx.simulate(lid, _params(w.params))
+    work, nign, _ = ctx.get_counters(sid, replicas)
+    few = ctx.simulate(lid, _params(dict(w.params, n_replicas=300)))
+    w300, n300, _ = ctx.get_counters(few, 300)
+    assert np.array_equal(work[:300], w300) and np.array_equal(nign[:300], n300)
+    for r in (0, 299):
+        for a, b in zip(ctx.get_replica_scar(sid, r, n, ign_steps=True), ctx.get_replica_scar(few, r, n, ign_steps=True)):
+            assert np.array_equal(a, b)
+    ctx.release(sid)
+    ctx.release(few)
+    ctx.release(lid)
