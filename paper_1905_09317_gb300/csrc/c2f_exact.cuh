@@ -142,6 +142,46 @@ C2F_HD double sqrt_mid(double x) {
   return double_of((uint64_t)q + ((uint64_t)((e + 1021u) >> 1) << 52));
 }
 
+// RN(x y) for x and y both positive in mid_range: the 128-bit product of the
+// significands, its dropped bits gathered in the last one kept
+C2F_HD double mul_mid(double x, double y) {
+  const uint64_t bx = bits_of(x), by = bits_of(y);
+  const uint32_t a1 = (uint32_t)(bx >> 21) | 0x80000000u, a0 = (uint32_t)(bx << 11);
+  const uint32_t b1 = (uint32_t)(by >> 21) | 0x80000000u, b0 = (uint32_t)(by << 11);
+  const uint64_t w0 = wide(a0, b0);
+  const uint64_t w1 = wide(a1, b0) + (w0 >> 32);
+  const uint64_t w2 = wide(a0, b1) + (uint32_t)w1;
+  uint64_t h = wide(a1, b1) + (w1 >> 32) + (w2 >> 32);            // [2^62, 2^64)
+  const uint32_t top = (uint32_t)(h >> 63);
+  h = (h << (1u - top)) | (((uint32_t)w0 | (uint32_t)w2) != 0u ? 1u : 0u);
+  uint64_t q = h >> 11;
+  q += ((uint32_t)h & 0x7FFu) + ((uint32_t)q & 1u) > 0x400u ? 1u : 0u;   // to nearest, ties to even
+  const uint32_t e = (uint32_t)(bx >> 52) + (uint32_t)(by >> 52) - 1024u + top;
+  return double_of(q + ((uint64_t)e << 52));
+}
+
+// 2^-500 <= x < 1
+C2F_HD bool below_one(uint64_t bits) { return (uint32_t)(bits >> 32) - (523u << 20) < (500u << 20); }
+
+// RN(1 - x) for x in below_one: in units of 2^-53 it is 2^53 less x rounded to
+// an integer when x < 1/2, and exact when x >= 1/2
+C2F_HD double one_minus(double x) {
+  const uint64_t b = bits_of(x);
+  const uint64_t m = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  uint32_t s = 1022u - (uint32_t)(b >> 52);                       // x = m 2^-(53 + s)
+  s = s > 60u ? 60u : s;                                          // far below 1/2: no integer part, no half
+  const uint64_t k = m >> s, rest = (m << 3) << (61u - s);         // rest: the fraction, as 64 bits
+  const bool up = rest > 0x8000000000000000ull || (rest == 0x8000000000000000ull && (k & 1u));
+  const uint64_t n = 0x20000000000000ull - k - (up ? 1u : 0u);
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)n);
+#else
+  const int lz = __builtin_clzll(n);
+#endif
+  const uint32_t left = lz > 11 ? (uint32_t)lz - 11u : 0u;
+  return double_of((n << left) + ((uint64_t)(1021u - left) << 52));
+}
+
 // ---- the Horner steps of exp and log
 // q = c + p r for a p of 53 bits and |r| < 2^-7, each sum rounded to binary64:
 // the exponents of every c and q are known ahead, so with r as a 64-bit integer

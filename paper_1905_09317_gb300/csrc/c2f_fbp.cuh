@@ -55,9 +55,10 @@ inline void make_fuel_table(FuelCoef t[F_NCODES]) {
 
 __device__ __forceinline__ bool is_o1(int f) { return f == F_O1A || f == F_O1B; }
 
+template <bool INTS>
 __device__ __forceinline__ double rsi_curve(const FuelCoef &k, double isi) {
-  const double x = __dsub_rn(1.0, dexp(__dmul_rn(-k.b, isi)));
-  return __dmul_rn(k.a, dpow_n2(x, k.c, k.c2));
+  const double x = done_minus<INTS>(dexp(-dmul_pos<INTS>(k.b, isi)));
+  return dmul_pos<INTS>(k.a, dpow_n2<INTS>(x, k.c, k.c2));
 }
 
 __device__ inline double curing_factor(double c) {
@@ -73,13 +74,14 @@ __device__ __forceinline__ int curve_of(int fuel, int i) { return curves_of(fuel
 // or (mixed woods) four times: a warp runs the whole of a cell-hour's 3,000
 // instructions from the instruction cache, and with every call inlined a
 // quarter of its stalls were instruction fetches.
+template <bool INTS>
 __device__ __forceinline__ void rsi_both(int fuel, double isi[2], double pcf, double cf) {
   const int nc = curves_of(fuel);
   double first = 0.0, x = isi[0], other = isi[1], done = 0.0;
 #pragma unroll 1
   for (int it = 0; it < 2 * nc; ++it) {
     const int i = nc == 2 ? it & 1 : 0;
-    const double v = rsi_curve(g_fuel[curve_of(fuel, i)], x);
+    const double v = rsi_curve<INTS>(g_fuel[curve_of(fuel, i)], x);
     if (i + 1 < nc) {
       first = __dmul_rn(pcf, v);
       continue;
@@ -157,7 +159,7 @@ __device__ inline void hour_prep(int f, double ws, double wd_from, double ffmc, 
   }
   double rz = 0.0;
   if (f != F_NONE && f != F_M1 && f != F_M2) {
-    rz = rsi_curve(g_fuel[f], isz);
+    rz = rsi_curve<false>(g_fuel[f], isz);
     if (is_o1(f)) rz = __dmul_rn(rz, cf);
   }
   hp->be[f] = be;
@@ -221,6 +223,7 @@ __device__ __forceinline__ double halved(double x) {
 // its rate along each of the 8 axes for the head direction (ux, uy) (unit
 // vector, x east, y north) by Eq. (1) (ellipse_mode 0) or by the ray from the
 // ignition point (mode 1).
+template <bool INTS>
 __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb, double ux, double uy,
                                              int ellipse_mode, AxisRates *o) {
   const double hb = __dadd_rn(hros, bros);
@@ -246,7 +249,7 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
       const uint64_t c = bits_of(c0);
       const double ahead = double_of(c & 0x7FFFFFFFFFFFFFFFull);
       o->behind |= (uint32_t)(c >> 63) << j;
-      const double q = pos(ahead) ? ddiv(A, __dsub_rn(1.0, __dmul_rn(e, ahead))) : A;
+      const double q = pos(ahead) ? ddiv(A, done_minus<INTS>(dmul_pos<INTS>(e, ahead))) : A;
       c0 = c1; c1 = c2; c2 = c3;   // the next axis' cosine, in registers
       r0 = r1; r1 = r2; r2 = r3; r3 = q;
     }
@@ -287,7 +290,9 @@ __device__ __forceinline__ void ellipse_axes(double hros, double bros, double lb
 
 // per (cell, hour): FBP surface spread, Eqs. (2)-(4), then the 8 axis rates
 // by Eq. (1) (ellipse_mode 0) or by the centre-offset ellipse ray (mode 1).
-__device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const HourPrep &hp,
+// INTS: see dmul_pos.
+template <bool INTS>
+__device__ __forceinline__ void fbp_row(int fuel, double gs, const CellPrep &cp, const HourPrep &hp,
                                double pcf, int ellipse_mode, AxisRates *o) {
   const double cf = hp.cf;
   double wse = 0.0;
@@ -316,7 +321,7 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
   double fw, fb;
   wind_fn(wsv, &fw, &fb);
   double rsi[2] = {__dmul_rn(hp.isz, fw), __dmul_rn(hp.isz, fb)};
-  rsi_both(fuel, rsi, pcf, cf);
+  rsi_both<INTS>(fuel, rsi, pcf, cf);
   const double be = hp.be[fuel];
   const double hros = __dmul_rn(rsi[0], be), bros = __dmul_rn(rsi[1], be);
   double lb;
@@ -324,7 +329,7 @@ __device__ inline void fbp_row(int fuel, double gs, const CellPrep &cp, const Ho
     lb = !lt_c(wsv, 1.0) ? __dmul_rn(1.1, dpow_n2(wsv, 0.464, 0)) : 1.0;
   else
     lb = __dadd_rn(1.0, __dmul_rn(8.729, dpow_n2(__dsub_rn(1.0, dexp(__dmul_rn(-0.030, wsv))), 2.155, 0)));
-  ellipse_axes(hros, bros, lb, ux, uy, ellipse_mode, o);
+  ellipse_axes<INTS>(hros, bros, lb, ux, uy, ellipse_mode, o);
 }
 
 // the integer nearest to x 2^up (ties to even) for a non-negative real, by

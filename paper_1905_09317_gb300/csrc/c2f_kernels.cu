@@ -208,13 +208,14 @@ __global__ void k_order_scatter(const uint8_t *fuel, const float *slope, const u
 // (const_ros > 0: the deterministic test rates -- all 8 axes at const_ros, or,
 // with const_bros > 0 or const_lb > 1, the ellipse of HROS = const_ros,
 // BROS = const_bros (0: const_ros), LB = const_lb headed along the hour's wind)
+template <bool INTS>
 __device__ __forceinline__ void row_rates(int fuel, const float *slope, int64_t cell,
                                           const CellPrep &cp, const HourPrep &hp, double pcf,
                                           double const_ros, double const_bros, double const_lb,
                                           int ellipse_mode, AxisRates *o) {
   if (pos(const_ros)) {
     if (pos(const_bros) || gt_c(const_lb, 1.0)) {
-      ellipse_axes(const_ros, pos(const_bros) ? const_bros : const_ros, gt_c(const_lb, 1.0) ? const_lb : 1.0,
+      ellipse_axes<INTS>(const_ros, pos(const_bros) ? const_bros : const_ros, gt_c(const_lb, 1.0) ? const_lb : 1.0,
                    hp.sin_w, hp.cos_w, ellipse_mode, o);
       return;
     }
@@ -224,7 +225,7 @@ __device__ __forceinline__ void row_rates(int fuel, const float *slope, int64_t 
     for (int k = 0; k < 8; ++k) o->ros[k] = const_ros;
     return;
   }
-  fbp_row(fuel, slope ? (double)slope[cell] : 0.0, cp, hp, pcf, ellipse_mode, o);
+  fbp_row<INTS>(fuel, slope ? (double)slope[cell] : 0.0, cp, hp, pcf, ellipse_mode, o);
 }
 
 // a table row: the 8 per-period increments B_k = fixed(ros_k * dt * 2^32) in one
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(128) k_ros_table(RosTableArgs a) {
   const size_t idx = (size_t)h * n + cell;
   AxisRates o;
   if (burn) {
-    row_rates(a.fuel[cell], a.slope, cell, a.cell[cell], a.hour[h], a.pcf, a.const_ros, a.const_bros, a.const_lb,
+    row_rates<true>(a.fuel[cell], a.slope, cell, a.cell[cell], a.hour[h], a.pcf, a.const_ros, a.const_bros, a.const_lb,
               a.ellipse_mode, &o);
     if (a.base) row_store(a.base + idx * 8, a.hros + idx, o, a.dt2p32);
   } else if (a.base) {
@@ -422,7 +423,7 @@ __device__ __forceinline__ void table_chunk(const SimJob &J, int32_t h, int32_t 
     const int64_t n = (int64_t)J.rows * J.cols;
     const int64_t cell = (int64_t)row * J.cols + col;
     AxisRates o;
-    row_rates(__ldg(&J.fuel[cell]), J.slope, cell, J.cell[cell], J.hour[h], J.pcf, J.const_ros, J.const_bros,
+    row_rates<false>(__ldg(&J.fuel[cell]), J.slope, cell, J.cell[cell], J.hour[h], J.pcf, J.const_ros, J.const_bros,
               J.const_lb, J.ellipse_mode, &o);
     const size_t idx = (size_t)h * n + cell;
     row_store(J.base + idx * 8, J.hros + idx, o, J.dt2p32);

@@ -122,6 +122,23 @@ __device__ __noinline__ double dexp_far(double x) {   // |x| >= 704 and not in (
 __device__ __forceinline__ double ddiv(double x, double y) {
   return mid_range(bits_of(x)) && mid_range(bits_of(y)) ? div_mid(x, y) : ddiv_any(x, y);
 }
+// x y for x, y >= 0 and 1 - x for 0 <= x <= 1: with INTS on the integer units,
+// too, else by the FP64 instructions.  The integer forms take some 40
+// instructions for one, so they pay only where the FP64 pipe is the bound and
+// their code runs from a loop: in the table kernel's curve and axis loops (512^2
+// x 24 h: 1.557 -> 1.490 ms; everywhere in that kernel 1.586 ms; in the
+// frontier's on-demand rows, which are bound by latency, 24.4 -> 26.7 ms).
+__device__ __noinline__ double done_minus_any(double x) { return __dsub_rn(1.0, x); }
+template <bool INTS>
+__device__ __forceinline__ double dmul_pos(double x, double y) {
+  if (!INTS) return __dmul_rn(x, y);
+  return mid_range(bits_of(x)) && mid_range(bits_of(y)) ? mul_mid(x, y) : dmul_any(x, y);
+}
+template <bool INTS>
+__device__ __forceinline__ double done_minus(double x) {
+  if (!INTS) return __dsub_rn(1.0, x);
+  return below_one(bits_of(x)) ? one_minus(x) : done_minus_any(x);
+}
 __device__ __forceinline__ double droot(double x) { return mid_range(bits_of(x)) ? sqrt_mid(x) : dsqrt_any(x); }
 
 // a binary32 integer as binary64, by its bits
@@ -287,16 +304,17 @@ __device__ __noinline__ double dpow_any(double x, double y) {   // x not positiv
   return __longlong_as_double(0x7ff8000000000000LL);
 }
 
-__device__ inline double dpow_n2(double x, double y, int n2) {
+template <bool INTS = false>
+__device__ __forceinline__ double dpow_n2(double x, double y, int n2) {
   if (!pos(x)) return dpow_any(x, y);
   if (n2 == 0) return dexp(__dmul_rn(y, dlog(x)));
   const int n = n2 >> 1;
   double r = x;
 #pragma unroll 1
-  for (int i = 1; i < n; ++i) r = __dmul_rn(r, x);
+  for (int i = 1; i < n; ++i) r = dmul_pos<INTS>(r, x);
   if (n2 & 1) {
     const double root = droot(x);
-    r = n > 0 ? __dmul_rn(r, root) : root;
+    r = n > 0 ? dmul_pos<INTS>(r, root) : root;
   }
   return r;
 }

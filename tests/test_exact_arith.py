@@ -30,6 +30,13 @@ extern "C" void steps(const double *r, long n, int log, double *q, double *e, un
       e[i] = std::fma(std::fma(std::fma(1.0 / 120, r[i], 1.0 / 24), r[i], 1.0 / 6), r[i], 0.5);
   }
 }
+extern "C" void products(const double *a, const double *b, long n, double *p, double *d, unsigned char *ok) {
+  for (long i = 0; i < n; ++i) {
+    p[i] = c2f::mul_mid(a[i], b[i]);
+    ok[i] = c2f::mid_range(c2f::bits_of(a[i])) && c2f::mid_range(c2f::bits_of(b[i]));
+    d[i] = c2f::below_one(c2f::bits_of(a[i])) ? c2f::one_minus(a[i]) : 1.0 - a[i];
+  }
+}
 extern "C" void run(const double *a, const double *b, long n, int ulps, double *q, double *s, unsigned char *ok) {
   g_scale = 1.0f + ulps * 0x1p-23f;
   for (long i = 0; i < n; ++i) {
@@ -97,3 +104,19 @@ def test_exp_and_log_steps_equal_fused_multiply_adds(lib):
         big = np.abs(r) > 2.0 ** -17.9
         assert use[big & ((r > 0) | (which == 0))].mean() > 0.999
         assert np.array_equal(q[use], e[use])
+
+
+@pytest.mark.parametrize("span", [1, 499])
+def test_product_and_one_minus_are_correctly_rounded(lib, span):
+    rng = np.random.default_rng(span)
+    n = 400_000
+    a, b = _values(rng, n, span), _values(rng, n, span)
+    a[: n // 2] = np.where(rng.random(n // 2) < 0.5, 1.0 - np.ldexp(rng.random(n // 2), -rng.integers(0, 53, n // 2)),
+                           np.ldexp(1.0 + np.round(rng.random(n // 2) * 8) / 8, -rng.integers(1, 60, n // 2)))
+    p, d, ok = np.empty(n), np.empty(n), np.empty(n, dtype=np.uint8)
+    lib.products(a.ctypes.data_as(C.c_void_p), b.ctypes.data_as(C.c_void_p), C.c_long(n), p.ctypes.data_as(C.c_void_p),
+                 d.ctypes.data_as(C.c_void_p), ok.ctypes.data_as(C.c_void_p))
+    use = ok.astype(bool)
+    assert use.mean() > 0.9
+    assert np.array_equal(p[use], (a * b)[use])
+    assert np.array_equal(d, 1.0 - a)
