@@ -1661,10 +1661,13 @@ __device__ __forceinline__ void count_cells4(const int4 &a, const int4 &b, int32
 // later of the two (cells both runs ignite), then prefix sums over hours give
 // a, b, c of every hour's scars; one pass over the two ignition-step arrays,
 // streamed with 16-byte loads (when the rows are aligned), four per array in
-// flight per thread.  128-thread CTAs so that every replica of a launch is
-// resident at once.  Dynamic shared memory: 3 H counters.  The final scars are
+// flight per thread.  HBM-bound, given enough threads in flight: CTAs of 128 to
+// 1,024 threads, as many as keep every replica of the launch resident at once
+// (500 pairs of 512 x 512: 287 us with 128 threads, 186 us, 5.6 TB/s, with 512;
+// 100 pairs 252 and, with 1,024, 60 us; a cluster of CTAs a replica was slower
+// than 128 threads).  Dynamic shared memory: 3 H counters.  The final scars are
 // the scars of the last hour, so ||X - Y|| comes from the same counts.
-__global__ void __launch_bounds__(128) k_compare_hours(const int32_t *__restrict__ step_x,
+__global__ void __launch_bounds__(1024) k_compare_hours(const int32_t *__restrict__ step_x,
                                                        const int32_t *__restrict__ step_y, int64_t n,
                                                        int32_t sph, int32_t H, double *mse, double *ssim,
                                                        double *dnorm) {

@@ -1822,7 +1822,11 @@ int compare_launch(c2f_ctx *ctx, int32_t sim_x, int32_t sim_y, double *mse, doub
     const size_t smem = sizeof(uint32_t) * 3 * (size_t)H;
     if (smem > 48 * 1024) CK(cudaFuncSetAttribute(k_compare_hours, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)smem));
-    k_compare_hours<<<R, 128, smem, st>>>(X->ign_step.as<int32_t>(), Y->ign_step.as<int32_t>(), X->n,
+    // 128 to 1,024 threads: all replicas resident at once (2,048 threads an SM),
+    // 16 cells or more a thread
+    int threads = 1024;
+    while (threads > 128 && ((int64_t)R * threads > (int64_t)ctx->sm_count * 2048 || (int64_t)threads * 16 > X->n)) threads /= 2;
+    k_compare_hours<<<R, threads, smem, st>>>(X->ign_step.as<int32_t>(), Y->ign_step.as<int32_t>(), X->n,
                                           60 / X->p.minutes_per_step, H, mse, ssim, dnorm);
     CKL("k_compare_hours");
   } else if (dnorm) {   // no hourly metrics asked for: the final scars' bit planes
