@@ -740,13 +740,13 @@ def roofline_table(kt, w, fp64_peak):
 # flops per cell-hour (2 x DFMA + DMUL + DADD from ncu's instruction counts over
 # cells x hours).  FP64 peak: 152 SMs x 2 DFMA per clock x 2 flop x 2.07 GHz.
 FRONTIER_BYTES_PER_UPDATE = 194.0
-FRONTIER_DRAM_BYTES_PER_REPLICA = (96.998e6 + 14.878e6) / 200   # 200-replica launch: read + write
-FRONTIER_WARP_INST_PER_UPDATE = 214.105e6 / 43484764             # warp instructions / cell-updates
-FRONTIER_L2_BYTES_PER_REPLICA = 20432252 * 32 / 200                 # lts__t_sectors x 32 B / replicas
-FRONTIER_L2_PCT_IN_CAPTURE = 0.43                                   # lts__t_sectors % of peak, same capture
+FRONTIER_DRAM_BYTES_PER_REPLICA = (98.203e6 + 3.330e6) / 200    # 200-replica launch: read + write
+FRONTIER_WARP_INST_PER_UPDATE = 96.512e6 / 43484764              # warp instructions / cell-updates
+FRONTIER_L2_BYTES_PER_REPLICA = 17912819 * 32 / 200                 # lts__t_sectors x 32 B / replicas
+FRONTIER_L2_PCT_IN_CAPTURE = 0.74                                   # lts__t_sectors % of peak, same capture
 FRONTIER_PROFILE_NOTE = "ncu dram__bytes_read+write and smsp__inst_executed of a 200-replica launch, " \
                         "scaled by replicas / cell-updates"
-FP64_OPS_PER_CELL_HOUR = 364.0      # ncu: (2 x DFMA + DMUL + DADD) / (cells x hours)
+FP64_OPS_PER_CELL_HOUR = 150.8      # ncu: (2 x DFMA + DMUL + DADD) / (cells x hours); the rest is integer arithmetic
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07   # SMs x DFMA/clk x flop/DFMA x GHz
 
 
