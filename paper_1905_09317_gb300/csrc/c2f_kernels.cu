@@ -668,7 +668,11 @@ __device__ __forceinline__ void help_with_chunks(const ChunkWork *work) {
 // of its 1,090 visited periods, most of them in passes that few lanes had work
 // for; a window holds 5 to 6 periods there, 25 entries, 18 crossings and 15 new
 // cells.  1,000 replicas: 4.42 ms one period at a time, 2.02 to 2.29 ms now;
-// 64 replicas 1.96 ms.
+// 64 replicas 1.96 ms.  Where a period takes dozens of windows (uniform fuel at a
+// constant rate: rings of hundreds of cells), scanning the list from its start
+// and compacting it before every window would grow with its square: 4 replicas,
+// 1500 x 1500 at 60 m/min for 24 h: 3.63 s so, 0.66 s with scan0 and room below
+// (one period at a time: 1.32 s); 2,000 replicas, 200 x 200 at 99: 113, 29 (81) ms.
 //
 // HELPERS warps of the CTA beside the frontier's own only compute on-demand
 // table rows (with WPC = 1; `work` in shared memory).
@@ -1117,18 +1121,30 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *
       W += (long long)dying * s0;
 
       // ---- the periods of this hour at which some axis reaches a centre
+      // scan0: where A1 starts.  Not 0 only with width 1, when this period has
+      // been begun: no entry before it crosses in it any more
+      int32_t scan0 = 0;
+      int32_t room = compact_at;   // compact above this many entries
       while (cal != 0ull) {
         const int32_t o1 = __ffsll((long long)cal) - 1;
         if (prof && lane == 0) { pc_t = clock64(); pq[7] = max(pq[7], (long long)cnt); }
-        if (cnt > compact_at) {   // keep room for new cells
+        // keep room for new cells.  Again only when half of the room that a
+        // compaction left is used up: a dense period has dozens of windows, and
+        // a list of mostly live entries would be compacted before each
+        // Not in an hour's first period with the threshold: cells that burn out
+        // at the boundary still send in it
+        if (cnt > room && (o1 > 0 || !use_delta)) {
           compact(cnt);
+          scan0 = 0;
+          room = max(compact_at, cnt + (cap - cnt) / 2);
           if (prof && lane == 0) pq[9] += 1;
         }
         const int32_t Ew = min(o1 + width, sph);   // the window is [o1, Ew), shortened below
         // (A1) the entries that cross in the window, up to 64
         int32_t got = 0;
         bool full = false;
-        for (int32_t g0 = 0; g0 < cnt && !full; g0 += 1024) {
+        int32_t g0 = scan0;
+        for (; g0 < cnt && !full; g0 += 1024) {
           uint32_t w = 0;   // bit 8 b + 7 - j: byte b of this lane's j-th word crosses
 #pragma unroll 2
           for (int j = 0; j < 8; ++j) {
@@ -1158,7 +1174,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *
         }
         got = min(got, 64);
         if (prof && lane == 0) pq[8] += clock64() - pc_t;
-        if (got == 0) { cal &= ~(1ull << o1); continue; }   // its entries were dropped by a compaction
+        if (got == 0) { cal &= ~(1ull << o1); scan0 = 0; continue; }   // its entries were dropped by a compaction
         // (A2) their crossings in the window towards Available cells, up to
         // 32: target cell into buf, offset into obuf
         bool broken = false, more = false;   // more: more than 32 crossings
@@ -1393,6 +1409,7 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *
         if (!full) cal &= ~((1ull << E) - 1ull);   // E <= 60
         uint64_t seen = 0;      // profile: periods at which a crossing was processed, entries with one
         int32_t crossed = 0;
+        uint32_t rest = full ? (uint32_t)(g0 - 1024) : 0xFFFFFFFFu;   // the first entry that may still cross before E
 #pragma unroll 1
         for (int32_t i0 = 0; i0 < got; i0 += 32) {
           bool closed = false;
@@ -1412,8 +1429,10 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *
               *at = v;
               enx[e] = (uint8_t)nx;
               bits |= cal_bit(nx);
+              if ((int32_t)nx < E) rest = min(rest, (uint32_t)e);
             } else if (more) {
               bits |= 1ull << o1;
+              rest = min(rest, (uint32_t)e);
             }
             if (PROF && closed)
               for (int j = 0; j < 8; ++j) {
@@ -1445,6 +1464,15 @@ __device__ __forceinline__ void frontier_warp(const FrontierArgs &A, ChunkWork *
         // the next window: as long as should fill it, a little longer than what this one reached
         width = min(max(1, (Ew - o1) * kWindowFill / got), E < Ew ? E - o1 + 2 : 32);
         width = min(width, 32);
+        if (scan0 > 0) width = 1;   // the end of a long period says nothing of the next one's density
+        scan0 = 0;
+        if (full || more) {         // one period, not done yet: on from its first entry that is left
+          rest = __reduce_min_sync(FULL, rest);
+          if (rest != 0xFFFFFFFFu) {
+            scan0 = (int32_t)(rest & ~1023u);
+            width = 1;
+          }
+        }
         __syncwarp();
         if (live == 0) break;
       }

@@ -159,3 +159,38 @@ def test_crowded_launches_equal_small_ones(ctx, replicas):
     ctx.release(sid)
     ctx.release(few)
     ctx.release(lid)
+
+
+@pytest.mark.parametrize("smem", [1, 0])
+@pytest.mark.parametrize("capacity", [0, 300, 2100])   # default; retried at four times as many; nearly full of live entries
+@pytest.mark.parametrize("over", [
+    dict(const_ros=100.0),                   # rings of up to 660 cells ignite in one period
+    dict(const_ros=60.0, ros_sigma=0.4, burnout_delta=30.0),   # some burn out at each hour's start
+    dict(const_ros=60.0, ros_sigma=0.3),     # up to 348 cells in one period
+])
+def test_periods_of_many_windows_equal_the_oracle(ctx, over, capacity, smem):
+    """Lists of more than one scan round (1,024 entries) whose periods take many windows, and compactions among them."""
+    rows, cols, hours = 330, 340, 3
+    fuel = np.full((rows, cols), 3, dtype=np.uint8)
+    weather = S.constant_weather(hours)
+    d = dict(dict(seed=5, n_replicas=1, hours=hours, minutes_per_step=1, ignition_mode=0,
+                  ignition_cell=165 * cols + 170, ros_sigma=0.0), **over)
+    ctx.set_frontier_config(32, smem)
+    ctx.set_list_capacity(capacity)
+    lid = ctx.load_landscape(fuel)
+    ctx.set_weather(lid, weather)
+    try:
+        sid = ctx.simulate(lid, _params(d))
+        _, ign = ctx.get_scars(sid, 1, fuel.size, ign_steps=True)
+        work, nign, _ = ctx.get_counters(sid, 1)
+        ctx.release(sid)
+    finally:
+        ctx.set_frontier_config(32, 1)
+        ctx.set_list_capacity(0)
+        ctx.release(lid)
+    z = np.zeros(fuel.shape, dtype=np.float32)
+    o = oracle.Oracle(fuel, z, z, cell_size=100.0, weather=weather, **d)
+    ref = o.run_replica(0)
+    o.close()
+    assert np.array_equal(ign[0], ref["ign"].ravel())
+    assert work[0] == ref["work"] and nign[0] == ref["n_ignited"]
